@@ -51,6 +51,7 @@ struct Bucket {
     int first, count;
     size_t off;           // workspace offset of the bucket's slot region
     int64_t inst_bytes;   // slot region of one instance
+    size_t dig_off;       // float64: digit buffers of the bucket's instances
 };
 
 struct Group {           // instances [i0, i1) with buckets [b0, b0 + nb): one grouped launch
@@ -82,6 +83,9 @@ struct Plan {
     std::vector<GramGroup> gram_grp;
     GramGeom gram_geom{};
     HostWork wg, wsc, we, wr, wgr, wct, wtc[2], wf64;   // wtc[0]: 256-wide tiles, wtc[1]: 128-wide
+    bool digits = false;      // float64 products on the tensor cores (gemm_digits.cu)
+    HostWork wdig;            // their units
+    std::vector<unsigned char> dig_maps;   // 128 bytes per bucket
     int tile_n = 0;
     int tile_ctas = 0;
     int tile_drain = 0;
@@ -300,8 +304,9 @@ bool plan_km(int n_terms, int k_req, int* k, int* m) {
 
 int split_count(int prec) { return prec == FO_PREC_BF16X3 ? 6 : (prec == FO_PREC_FP16X2 ? 3 : 1); }
 
-// Shape, sort order, buckets and the workspace layout (offsets only).
-fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p) {
+// Shape, sort order, buckets and the workspace layout (offsets only). digits: whether a float64
+// plan may hold the digit buffers of the tensor-core products.
+fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     const int batch = (int)key.n.size();
     if (batch < 1) return fail(ctx, FO_ERR_ARG, "batch must be >= 1");
     for (int64_t n : key.n) {
@@ -375,13 +380,30 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p) {
         const size_t np2 = (size_t)np * (size_t)np;
         in.slot_bytes = (int64_t)(sh.is64 ? align256(np2 * 8) : align256(np2 * 4 + (size_t)sh.planes * np2 * 2));
         if (p->buckets.empty() || p->buckets.back().np != np) {
-            Bucket bk{np, j, 0, 0, (int64_t)in.slot_bytes * p->n_slots};
+            Bucket bk{np, j, 0, 0, (int64_t)in.slot_bytes * p->n_slots, 0};
             p->buckets.push_back(bk);
         }
         in.bucket = (int)p->buckets.size() - 1;
         in.in_bucket = p->buckets.back().count++;
     }
     for (Bucket& bk : p->buckets) bk.off = take((size_t)bk.inst_bytes * bk.count);
+    // float64 plans whose chains run step by step: digit buffers (staged chains multiply arbitrary
+    // pairs of slots and keep the FMA kernel)
+    p->digits = digits && sh.is64 && !key.staged && (key.mode == MODE_DENSITY || key.mode == MODE_MOMENTS);
+    if (p->digits) {
+        std::vector<int64_t> ns, nps;
+        for (const Inst& in : p->inst) {
+            ns.push_back(in.n);
+            nps.push_back(in.np);
+        }
+        std::vector<int> sl(batch), sh_(batch);
+        dig_splits(ns.data(), nps.data(), batch, std::max(1, ctx->num_sms), sl.data(), sh_.data());
+        for (int j = 0; j < batch; ++j) {
+            p->inst[j].dig_sl = sl[j];
+            p->inst[j].dig_sh = sh_[j];
+        }
+        for (Bucket& bk : p->buckets) bk.dig_off = take((size_t)kDigBufs * 16 * bk.np * bk.np * bk.count);
+    }
     // per-instance float64 arrays
     std::vector<size_t> small(batch);
     const int ndiag = sh.n_tslots + 2;
@@ -398,6 +420,12 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p) {
         o += align256(8 * (size_t)p->npairs);         // gram
         o += align256(8 * (size_t)p->npairs * in.gram_blocks);   // gram partials
         o += align256(8 * (3 * (size_t)in.np + 2 * kLzMax + 3));  // Lanczos state
+        if (p->digits) {
+            o += align256(8 * (size_t)p->n_slots);                          // smax
+            o += align256(4 * (size_t)p->n_slots * kDigMaxSplit);           // umax
+            o += align256(4 * (size_t)p->n_slots);                          // sexp
+            o += align256(8 * 16384 * (size_t)dig_units(in.np, in.dig_sl, in.dig_sh));   // unit sums
+        }
         small[j] = off;
         off = o;
     }
@@ -417,6 +445,7 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p) {
     fill(p->wtc[0], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 256) : tc_tiles(in.np, 256); });
     fill(p->wtc[1], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 128) : tc_tiles(in.np, 128); });
     fill(p->wf64, [](const Inst& in) { return f64_tiles(in.np); });
+    fill(p->wdig, [&](const Inst& in) { return p->digits ? dig_units(in.np, in.dig_sl, in.dig_sh) : int64_t(0); });
     const size_t off_pg = take(8 * 3 * (size_t)std::max(1, p->wg.pre[batch]));
     const size_t off_pt = take(8 * 2 * (size_t)std::max(1, p->wr.pre[batch]));
     const size_t off_ptc = take(8 * 2 * (size_t)std::max(1, p->wtc[1].pre[batch]));   // 128-blocks
@@ -478,12 +507,20 @@ fo_status place_plan(fo_ctx* ctx, Plan* p) {
         in.gram = next(8 * (size_t)p->npairs);
         in.gpart = next(8 * (size_t)p->npairs * in.gram_blocks);
         in.lz = next(8 * (3 * (size_t)in.np + 2 * kLzMax + 3));
+        if (p->digits) {
+            in.dig = W + bk.dig_off + (size_t)kDigBufs * 16 * in.np * in.np * in.in_bucket;
+            in.smax = reinterpret_cast<unsigned long long*>(next(8 * (size_t)p->n_slots));
+            in.umax = reinterpret_cast<unsigned*>(next(4 * (size_t)p->n_slots * kDigMaxSplit));
+            in.sexp = reinterpret_cast<int32_t*>(next(4 * (size_t)p->n_slots));
+            in.dpart = reinterpret_cast<long long*>(next(8 * 16384 * (size_t)dig_units(in.np, in.dig_sl, in.dig_sh)));
+        }
         in.res = p->d_res + j;
     }
     // device tables: Inst[batch], InstIO[batch], the prefix arrays, then the cosine table of
     // the coefficient nodes. These stay valid for the plan's life: the workspace is shared
     // by every cached plan of the context, and another plan's call overwrites it.
-    HostWork* lists[] = {&p->wg, &p->wsc, &p->we, &p->wr, &p->wgr, &p->wct, &p->wtc[0], &p->wtc[1], &p->wf64};
+    HostWork* lists[] = {&p->wg,  &p->wsc,    &p->we,     &p->wr,   &p->wgr,
+                         &p->wct, &p->wtc[0], &p->wtc[1], &p->wf64, &p->wdig};
     size_t bytes = align256(sizeof(Inst) * batch) + align256(sizeof(InstIO) * batch);
     for (HostWork* w : lists) bytes += align256(sizeof(int) * w->pre.size());
     const size_t off_ct = bytes;
@@ -524,13 +561,23 @@ fo_status place_plan(fo_ctx* ctx, Plan* p) {
                     return fail(ctx, FO_ERR_CUDA, "tensor map: " + err);
         }
     }
+    if (p->digits) {
+        p->dig_maps.assign(128 * p->buckets.size(), 0);
+        for (size_t b = 0; b < p->buckets.size(); ++b) {
+            const Bucket& bk = p->buckets[b];
+            std::string err;
+            if (!dig_make_map(p->dig_maps.data() + 128 * b, W + bk.dig_off, bk.np, bk.count,
+                              (int64_t)kDigBufs * 16 * bk.np * bk.np, &err))
+                return fail(ctx, FO_ERR_CUDA, "digit tensor map: " + err);
+        }
+    }
+    p->gram_grp.clear();
+    for (const Group& g : p->groups) p->gram_grp.push_back(GramGroup{g.b0, g.nb, g.i0, g.i1});
     // geometry of the float32 masters for the Frobenius products' tensor maps
     if (!sh.is64 && p->n_slots > 0) {
         p->gram_bk.clear();
         for (const Bucket& bk : p->buckets)
             p->gram_bk.push_back(GramBucket{W + bk.off, bk.np, p->inst[bk.first].slot_bytes, bk.inst_bytes, bk.count});
-        p->gram_grp.clear();
-        for (const Group& g : p->groups) p->gram_grp.push_back(GramGroup{g.b0, g.nb, g.i0, g.i1});
         p->gram_geom = GramGeom{p->gram_bk.data(), p->gram_grp.data(), (int)p->gram_grp.size(), p->n_slots,
                                 p->wgr.pre.data()};
     }
@@ -574,6 +621,9 @@ Step make_step(const Plan& p, int a, int b, int c, int d, int out, double alpha,
     return st;
 }
 
+// Digit buffer of a slot of a float64 plan (see kDigBufs).
+int dig_buf(const Plan& p, int slot) { return slot == 0 ? 0 : (slot < p.sh.k ? 1 : 2); }
+
 // Independent products of the whole batch (one stage), at most kMaxSteps per launch.
 fo_status run_products(fo_ctx* ctx, Plan& p, const Step* steps, int nsteps, cudaStream_t s, const char* tag,
                        int index, Run* run, int prec = -1) {
@@ -584,7 +634,21 @@ fo_status run_products(fo_ctx* ctx, Plan& p, const Step* steps, int nsteps, cuda
         const int nq = std::min(kMaxSteps, nsteps - q0);
         const int h = prof_begin(ctx, s, FO_STAGE_PRODUCTS);
         int launches = 0;
-        if (p.sh.is64) {
+        if (p.digits) {
+            for (int q = q0; q < q0 + nq; ++q) {
+                // the result's digits: every slot is the next step's operand (the last giant step's,
+                // and P's, are not needed)
+                const Step& st = steps[q];
+                const bool last_giant = st.out >= p.sh.k && st.out == p.sh.n_tslots - 1;
+                // Gershgorin bounds enclose the spectrum; given and Lanczos bounds may not
+                const bool enclosed = !st.out64 && st.out < p.sh.n_tslots && !p.key.use_given && p.key.lanczos == 0;
+                const int dout = st.out64 || last_giant ? -1 : dig_buf(p, st.out);
+                FO_CUDA(dig_product(st, dig_buf(p, st.a), dig_buf(p, st.b), dout, p.d_inst, p.d_io, p.wdig.dev,
+                                    p.wdig.pre.data(), p.wsc.dev, p.gram_grp.data(),
+                                    (int)p.gram_grp.size(), p.dig_maps.data(), enclosed, ctx->flag, s, &launches),
+                        "dig_product");
+            }
+        } else if (p.sh.is64) {
             FO_CUDA(launch_gemm_f64(steps + q0, nq, p.d_inst, p.d_io, p.wf64.dev, s), "gemm_f64");
             launches = 1;
         } else {
@@ -778,14 +842,23 @@ fo_status clenshaw(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run) {
     return run_chain(ctx, p, chain, s, "clenshaw", run);
 }
 
+// X into slot 0 (float64 plans on the tensor cores: and its digits).
+fo_status scaled_x(fo_ctx* ctx, Plan& p, cudaStream_t s, int* launches) {
+    if (p.digits) FO_CUDA(dig_reset(p.d_inst, p.batch, 0, p.sh.n_tslots, s), "digit records");
+    FO_CUDA(launch_scale(p.d_inst, p.d_io, p.wsc.dev, p.sh, s, ctx->flag + 1), "scale");
+    if (p.digits) FO_CUDA(dig_split(p.d_inst, p.wsc.dev, 0, 0, 0, s), "digits of X");
+    *launches += p.digits ? 3 : 1;
+    return FO_OK;
+}
+
 // Spectral bounds, X and the baby steps T_2..T_k of every instance.
 fo_status front(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run) {
     const int h = prof_begin(ctx, s, FO_STAGE_BOUNDS);
     FO_CUDA(launch_bounds(p.d_inst, p.d_io, p.batch, p.wg.dev, p.part_g, p.key.use_given, s), "bounds");
-    int l = (p.key.use_given ? 1 : 2) + 1;
+    int l = p.key.use_given ? 1 : 2;
     if (p.key.lanczos > 0 && !p.key.use_given)
         FO_CUDA(launch_lanczos(p.d_inst, p.d_io, p.batch, p.wg.dev, p.part_g, p.key.lanczos, s, &l), "lanczos");
-    FO_CUDA(launch_scale(p.d_inst, p.d_io, p.wsc.dev, p.sh, s, ctx->flag + 1), "scale");
+    FO_TRY(scaled_x(ctx, p, s, &l));
     prof_end(ctx, s, h, 0.0, l);
     run->launches += l;
     return baby_steps(ctx, p, p.sh.k, s, run);
@@ -872,7 +945,12 @@ fo_status evaluate(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int poly_trac
     run->launches += lstage;
     h = prof_begin(ctx, s, FO_STAGE_CONTRACT);
     lstage = sh.is64 ? 1 : (sh.m + 31) / 32 + (sh.m > 1 ? 1 : 0);   // + the plane mirror of R_{m-1}
+    if (p.digits && sh.m > 1) FO_CUDA(dig_reset(p.d_inst, p.batch, sh.n_tslots, sh.m, s), "digit records");
     FO_CUDA(launch_contract(p.d_inst, p.we.dev, p.wct.dev, p.wsc.dev, sh, s, ctx->flag + 1), "contract");
+    if (p.digits && sh.m > 1) {
+        FO_CUDA(dig_split(p.d_inst, p.wsc.dev, sh.n_tslots, sh.m, dig_buf(p, sh.n_tslots), s), "digits of R");
+        lstage += 2;
+    }
     if (sh.m == 1) {
         FO_CUDA(launch_copy_out(p.d_inst, p.d_io, p.we.dev, sh, s), "copy_out");
         lstage += 1;
@@ -1097,8 +1175,16 @@ fo_status get_plan(fo_ctx* ctx, const PlanKey& key, Plan** out) {
     }
     std::unique_ptr<Plan> p(new (std::nothrow) Plan());
     if (!p) return fail(ctx, FO_ERR_NOMEM, "plan allocation failed");
-    FO_TRY(layout_plan(ctx, key, p.get()));
-    FO_TRY(ensure_ws(ctx, p->total));
+    FO_TRY(layout_plan(ctx, key, p.get(), true));
+    fo_status ws = ensure_ws(ctx, p->total);
+    if (ws == FO_ERR_NOMEM && p->digits) {
+        // without the digit buffers the workspace may fit: the products then run the FMA kernel
+        p.reset(new (std::nothrow) Plan());
+        if (!p) return fail(ctx, FO_ERR_NOMEM, "plan allocation failed");
+        FO_TRY(layout_plan(ctx, key, p.get(), false));
+        ws = ensure_ws(ctx, p->total);
+    }
+    FO_TRY(ws);
     // stale plans (older workspace) and the least recently used beyond the cap
     bool stale = false;
     for (auto& q : ctx->plans) stale |= q->ws_gen != ctx->ws_gen;
@@ -1781,7 +1867,7 @@ fo_status fo_moments(fo_ctx* ctx, const double* dH, int64_t n, int64_t ld, const
     Run run;
     FO_CUDA(launch_set_io(&io, 1, p->d_io, p->d_inst, 0, st), "set_io");
     FO_CUDA(launch_bounds(p->d_inst, p->d_io, 1, p->wg.dev, p->part_g, 1, st), "bounds");
-    FO_CUDA(launch_scale(p->d_inst, p->d_io, p->wsc.dev, p->sh, st, ctx->flag + 1), "scale");
+    FO_TRY(scaled_x(ctx, *p, st, &run.launches));
     FO_TRY(baby_steps(ctx, *p, p->sh.k, st, &run));
     FO_TRY(exact_moments(ctx, *p, st, &run));
     FO_CUDA(cudaMemcpyAsync(d_tau, p->inst[0].tau, 8 * (size_t)n_moments, cudaMemcpyDeviceToDevice, st),

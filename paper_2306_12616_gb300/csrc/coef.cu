@@ -338,6 +338,9 @@ __global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ i
     const int64_t tstride = in.slot_bytes / 8;
     const double* tbase = reinterpret_cast<const double*>(in.slots);
     double* rbase = reinterpret_cast<double*>(in.slots + n_tslots * in.slot_bytes);
+    // bits of the largest |entry| of the last R, the scale of its digits
+    const int last = (in.res->m_eff > 0 ? in.res->m_eff : m) - 1;
+    unsigned long long mx = 0;
     for (int64_t idx = r0 * np + threadIdx.x; idx < r1 * np; idx += blockDim.x) {
         const int64_t r = idx / np, col = idx - r * np;
         const bool diag = (r == col) && (r < n);
@@ -357,10 +360,15 @@ __global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ i
                     double v = acc[q];
                     if (diag) v += gsh[(l0 + q) * k];
                     rbase[(int64_t)(l0 + q) * tstride + idx] = v;
+                    if (l0 + q == last) {
+                        const unsigned long long av = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+                        mx = av > mx ? av : mx;
+                    }
                 }
             }
         }
     }
+    if (in.smax) max_to(in.smax + n_tslots + last, mx);
 }
 
 // float32 version: slots hold a float32 master at element offset 0 and 16-bit planes at

@@ -1,6 +1,8 @@
-// Float64 recurrence product out = alpha * A B + beta * C + D + shift * I_n (plain path).
+// Float64 recurrence product out = alpha * A B + beta * C + D + shift * I_n on the float64 FMA pipe:
+// the float64 path of staged chains, and of plans whose digit buffers do not fit the device
+// (elsewhere gemm_digits.cu, 8 to 40 times faster at N = 256 ... 2000).
 //
-// tcgen05 has no float64 kind, so the float64 path runs on the DFMA pipe: 64 x 64 output
+// 64 x 64 output
 // tiles, 16-deep k slices staged in shared memory, 4 x 4 outputs per thread. The update of
 // the three-term recurrence (2 T_1 T_i - T_{i-1}) and of the Clenshaw giant steps
 // (2 Y b_{l+1} - b_{l+2} + R_l) is applied in the epilogue, so every step is one launch.

@@ -71,6 +71,13 @@ struct Inst {
     int32_t in_bucket;    // index within the bucket
     int32_t gram_blocks;  // blocks of the Frobenius-product kernel for this instance
     int32_t user;         // index of the instance in the caller's arrays
+    // float64 products on the tensor cores (gemm_digits.cu); null / 0 elsewhere
+    char* dig;            // kDigBufs digit buffers of 16 np^2 bytes
+    long long* dpart;     // exact sums of the product's units, 128 x 128 each
+    unsigned long long* smax;   // per slot: bits of the largest |entry|
+    unsigned* umax;       // per slot and k range: bound of the product's high-order sums (float bits)
+    int32_t* sexp;        // per slot: scale exponent of its digits
+    int32_t dig_sl, dig_sh;     // k ranges of the low- and high-order units
 };
 
 // Per-call inputs of an instance (written at the start of every call).
@@ -185,6 +192,16 @@ __device__ __forceinline__ void upper_tile(int b, int tn, int& bi, int& bj) {
     while (r + 1 < tn && P(r + 1) <= b) ++r;
     bi = r;
     bj = r + (b - P(r));
+}
+
+// Largest |v| of a full warp into *dst, b the bits of |v| (non-negative doubles order as integers,
+// a NaN above every number).
+__device__ __forceinline__ void max_to(unsigned long long* dst, unsigned long long b) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, b, o);
+        b = x > b ? x : b;
+    }
+    if ((threadIdx.x & 31) == 0 && b) atomicMax(dst, b);
 }
 
 // Asynchronous 16-byte global -> shared copies (cp.async, L2 only) and their group waits.
@@ -457,6 +474,33 @@ cudaError_t launch_gemm_f64(const Step* steps, int nsteps, const Inst* in, const
                             cudaStream_t s);
 
 constexpr int kMaxBuckets = 16;   // tensor maps per grouped launch
+
+// ------------------------------------------------------------------ gemm_digits.cu
+constexpr int kDigMaxSplit = 16;  // k ranges of one tile at most
+// Digit buffers of an instance: X = T_1; the baby step T_i in work and then Y = T_k; the giant
+// step or Clenshaw (Horner) member in work. A result overwrites the operand it replaces, after
+// the product that read it.
+constexpr int kDigBufs = 3;
+int64_t dig_units(int64_t np, int sl, int sh);
+// k ranges of the low- and high-order units per instance, for `sms` SMs.
+void dig_splits(const int64_t* n, const int64_t* np, int count, int sms, int* sl, int* sh);
+// 4-D tensor map (entry, row, buffer, instance) over a bucket's digit buffers: rows of np / 16
+// k16 blocks of 8 digits x 16 float16 entries; boxes of 64 entries (4 digits) x 128 rows.
+bool dig_make_map(void* map128, const void* base, int64_t np, int count, int64_t inst_bytes, std::string* err);
+// One product of the whole batch: the units (prefix wu, host copy pre_host) and the update.
+// enclosed: the result is a T_j(X) on bounds that enclose the spectrum (|entries| <= 1). dig_out: the
+// digit buffer of the result (-1: none).
+cudaError_t dig_product(const Step& s, int dig_a, int dig_b, int dig_out, const Inst* in, const InstIO* io,
+                        const Work& wu, const int* pre_host, const Work& wsym, const GramGroup* grp,
+                        int ngrp, const void* maps, bool enclosed, int* err_flag, cudaStream_t st, int* launches);
+// Digits of a slot (last_m > 0: of the last R, slot0 + its l) into buffer buf.
+cudaError_t dig_split(const Inst* in, const Work& wsym, int slot0, int last_m, int buf, cudaStream_t st);
+// Clears the records of slots [slot0, slot0 + count).
+cudaError_t dig_reset(const Inst* in, int batch, int slot0, int count, cudaStream_t st);
+// Tiled tensor map over 16-bit floats with 128-byte swizzle.
+bool encode_map_f16(void* map128, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                    const uint32_t* box, std::string* err);
+
 int64_t tc_tiles(int64_t np, int tile_n);
 int tc_planes(int prec);
 // 5-D tensor map over the planes of every slot of every instance of one bucket:

@@ -14,6 +14,7 @@
 #include "exactsum.h"
 #include "fpbits.h"
 #include "internal.cuh"
+#include "tcptx.cuh"
 
 namespace fo {
 namespace {
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ inst
     // each thread scales the entries it loaded (the lower half of a diagonal tile is never
     // read: it is written from the upper half); the diagonal's formula only in diagonal tiles
     // (a block-uniform test, so that the other tiles carry no float64 work for it)
+    unsigned long long mx = 0;   // bits of the largest |entry| (float64 plans: the scale of X's digits)
     for (int ry = ty; ry < 32; ry += 8) {
         const int64_t r = (int64_t)bi * 32 + ry, c = (int64_t)bj * 32 + tx;
         const bool in = r < n && c < n && (bi != bj || tx >= ry);
@@ -291,6 +293,8 @@ __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ inst
             double v = 0.0;
             if (in) v = dg ? (2.0 * tile[ry][tx] - csum) * inv : tile[ry][tx] * inv2;
             tile[ry][tx] = v;
+            const unsigned long long av = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+            mx = av > mx ? av : mx;
         } else {
             // float32 of the exact product in integer operations (the float64 multiply was
             // this kernel's bound on the narrow float64 pipe)
@@ -299,6 +303,7 @@ __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ inst
             tf[ry][tx] = f;
         }
     }
+    if (insts[i].smax) max_to(insts[i].smax, mx);
     __syncthreads();
     char* slot = insts[i].slots;
     double* X64 = reinterpret_cast<double*>(slot);
@@ -659,15 +664,6 @@ struct GramMaps {
     CUtensorMap g[kMaxBuckets];   // boxes of 128 columns x 1 row x ngiant slots
     CUtensorMap b[kMaxBuckets];   // boxes of 128 columns x 1 row x nbaby slots
 };
-
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
-                                            int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
 
 // (row, chunk of the row) of upper chunk c of an np x np matrix cut into kc-entry chunks
 __device__ __forceinline__ void upper_chunk_pos(int64_t c, int64_t np, int kc, int& row, int& cc) {
