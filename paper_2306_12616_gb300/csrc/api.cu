@@ -100,7 +100,7 @@ struct Plan {
     double* part_g = nullptr;
     double* part_t = nullptr;
     double* part_tc = nullptr;    // per-tile (tr, ||.||^2) partials of the float64-output products
-    float* lscratch = nullptr;    // learned mu: features, normalised features, activations, outputs
+    float* lscratch = nullptr;    // learned mu: features, outputs
     int* lcount = nullptr;        // learned mu: instances still active after a judge
     size_t total = 0;
     double flops_product = 0.0;   // algorithmic flops of one product over the batch
@@ -450,7 +450,7 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     const size_t off_pt = take(8 * 2 * (size_t)std::max(1, p->wr.pre[batch]));
     const size_t off_ptc = take(8 * 2 * (size_t)std::max(1, p->wtc[1].pre[batch]));   // 128-blocks
     const size_t off_cnt = take(4 * ((size_t)batch + 8));
-    const size_t off_ls = take(4 * (size_t)batch * (2 * kMlpIn + 4 * kMlpHidden + kMlpOut));
+    const size_t off_ls = take(4 * (size_t)batch * (kMlpIn + kMlpOut));
     const size_t off_lc = take(sizeof(int));
     p->total = off;
     // remember the offsets in the (not yet placed) pointers
@@ -974,12 +974,7 @@ fo_status propose(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int use_order)
     const float* params = ctx->mlp;
     const float* norm = ctx->mlp + 4 * (size_t)mo.total;
     float* feat = p.lscratch;
-    float* xn = feat + (size_t)B * kMlpIn;
-    float* z1 = xn + (size_t)B * kMlpIn;
-    float* a1 = z1 + (size_t)B * kMlpHidden;
-    float* z2 = a1 + (size_t)B * kMlpHidden;
-    float* a2 = z2 + (size_t)B * kMlpHidden;
-    float* y = a2 + (size_t)B * kMlpHidden;
+    float* y = feat + (size_t)B * kMlpIn;
     int h = prof_begin(ctx, s, FO_STAGE_MOMENTS);
     int l0 = run->launches;
     FO_CUDA(launch_diag_sums(p.d_inst, B, sh.k, sh, s), "diag_sums");
@@ -990,12 +985,11 @@ fo_status propose(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int use_order)
     prof_end(ctx, s, h, 0.0, run->launches - l0);
     h = prof_begin(ctx, s, FO_STAGE_MU);
     FO_CUDA(launch_features(p.d_inst, p.d_io, B, sh.k, 0, feat, s), "features");
-    FO_CUDA(mlp_gather_norm(feat, nullptr, B, kMlpIn, norm, norm + kMlpIn, xn, s), "normalise");
-    FO_CUDA(mlp_forward(params, xn, B, z1, a1, z2, a2, y, s), "network");
+    FO_CUDA(mlp_forward(params, feat, norm, B, y, s), "network");
     FO_CUDA(launch_learned_mu(p.d_inst, B, y, norm, sh.n_terms, sh.k, sh.m, use_order, kOrderMargin, s),
             "proposal");
-    prof_end(ctx, s, h, 0.0, 6);
-    run->launches += 6;
+    prof_end(ctx, s, h, 0.0, 3);
+    run->launches += 3;
     return FO_OK;
 }
 
@@ -1432,7 +1426,6 @@ fo_status density_batch(fo_ctx* ctx, int batch, const double* const* dH, const i
 // ---------------------------------------------------------------- learned model
 size_t mlp_floats() { return 4 * (size_t)mlp_offsets().total + kMlpNorm; }
 float* mlp_params(fo_ctx* ctx) { return ctx->mlp; }
-float* mlp_grad(fo_ctx* ctx) { return ctx->mlp + mlp_offsets().total; }
 float* mlp_m(fo_ctx* ctx) { return ctx->mlp + 2 * (size_t)mlp_offsets().total; }
 float* mlp_v(fo_ctx* ctx) { return ctx->mlp + 3 * (size_t)mlp_offsets().total; }
 float* mlp_norm(fo_ctx* ctx) { return ctx->mlp + 4 * (size_t)mlp_offsets().total; }
@@ -1992,12 +1985,7 @@ fo_status fo_mlp_forward(fo_ctx* ctx, const float* d_x, int32_t n, float* d_y, v
     if (!ctx->mlp_ready) return fail(ctx, FO_ERR_UNSUPPORTED, "no model");
     DeviceGuard g(ctx->device);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    FO_TRY(ensure_mlp_scratch(ctx, (size_t)n * 4 * kMlpHidden));
-    float* z1 = ctx->mlp_scratch;
-    float* a1 = z1 + (size_t)n * kMlpHidden;
-    float* z2 = a1 + (size_t)n * kMlpHidden;
-    float* a2 = z2 + (size_t)n * kMlpHidden;
-    FO_CUDA(mlp_forward(mlp_params(ctx), d_x, n, z1, a1, z2, a2, d_y, st), "network");
+    FO_CUDA(mlp_forward(mlp_params(ctx), d_x, nullptr, n, d_y, st), "network");
     return FO_OK;
 }
 
@@ -2007,20 +1995,17 @@ fo_status fo_mlp_gradients(fo_ctx* ctx, const float* d_x, const float* d_t, int3
     if (!ctx->mlp_ready) return fail(ctx, FO_ERR_UNSUPPORTED, "no model");
     DeviceGuard g(ctx->device);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t B = (size_t)n;
-    FO_TRY(ensure_mlp_scratch(ctx, B * (6 * kMlpHidden + 2 * kMlpOut) + 1));
-    float* z1 = ctx->mlp_scratch;
-    float* a1 = z1 + B * kMlpHidden;
-    float* z2 = a1 + B * kMlpHidden;
-    float* a2 = z2 + B * kMlpHidden;
-    float* dz2 = a2 + B * kMlpHidden;
-    float* dz1 = dz2 + B * kMlpHidden;
-    float* y = dz1 + B * kMlpHidden;
-    float* dy = y + B * kMlpOut;
-    float* loss = dy + B * kMlpOut;
-    FO_CUDA(mlp_forward(mlp_params(ctx), d_x, n, z1, a1, z2, a2, y, st), "network");
-    FO_CUDA(mlp_backward(mlp_params(ctx), d_x, d_t, n, z1, a1, z2, a2, y, dy, dz2, dz1, d_grad, loss, st),
-            "backward");
+    FO_TRY(ensure_mlp_scratch(ctx, mlp_step_floats(n) + 1));
+    float* loss = ctx->mlp_scratch + mlp_step_floats(n);
+    MlpStep ms{};
+    ms.params = mlp_params(ctx);
+    ms.feat = d_x;
+    ms.target = d_t;
+    ms.B = n;
+    ms.scratch = ctx->mlp_scratch;
+    ms.grad = d_grad;
+    ms.loss = loss;
+    FO_CUDA(mlp_step(ms, st), "gradients");
     if (h_loss) {
         FO_CUDA(cudaMemcpyAsync(h_loss, loss, sizeof(float), cudaMemcpyDeviceToHost, st), "loss");
         FO_CUDA(cudaStreamSynchronize(st), "sync");
@@ -2039,26 +2024,14 @@ fo_status fo_mlp_train(fo_ctx* ctx, const float* d_feat, const float* d_target, 
     const int B = batch < n ? batch : n;
     const int steps = (n + B - 1) / B;
     const size_t total_steps = (size_t)steps * epochs;
-    const size_t Bz = (size_t)B;
-    const size_t need = Bz * (kMlpIn + kMlpOut + 6 * kMlpHidden + 2 * kMlpOut) + total_steps + (size_t)n;
-    FO_TRY(ensure_mlp_scratch(ctx, need));
-    float* xb = ctx->mlp_scratch;
-    float* tb = xb + Bz * kMlpIn;
-    float* z1 = tb + Bz * kMlpOut;
-    float* a1 = z1 + Bz * kMlpHidden;
-    float* z2 = a1 + Bz * kMlpHidden;
-    float* a2 = z2 + Bz * kMlpHidden;
-    float* dz2 = a2 + Bz * kMlpHidden;
-    float* dz1 = dz2 + Bz * kMlpHidden;
-    float* y = dz1 + Bz * kMlpHidden;
-    float* dy = y + Bz * kMlpOut;
-    float* losses = dy + Bz * kMlpOut;
+    const size_t rows = mlp_step_floats(B);
+    FO_TRY(ensure_mlp_scratch(ctx, rows + total_steps + (size_t)n));
+    float* losses = ctx->mlp_scratch + rows;
     int* idx = reinterpret_cast<int*>(losses + total_steps);
     float* norm = mlp_norm(ctx);
     // normalisation from the training set
     FO_CUDA(mlp_col_stats(d_feat, n, kMlpIn, norm, norm + kMlpIn, st), "stats");
     FO_CUDA(mlp_col_stats(d_target, n, kMlpOut, norm + 2 * kMlpIn, norm + 2 * kMlpIn + kMlpOut, st), "stats");
-    const int P = mlp_offsets().total;
     std::vector<int> perm(n);
     uint64_t rs = seed ^ 0x5DEECE66Dull;
     size_t step_i = 0;
@@ -2071,18 +2044,21 @@ fo_status fo_mlp_train(fo_ctx* ctx, const float* d_feat, const float* d_target, 
         FO_CUDA(cudaStreamSynchronize(st), "sync");
         FO_CUDA(cudaMemcpy(idx, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice), "order");
         for (int j = 0; j < steps; ++j, ++step_i) {
-            const int Bj = (j + 1) * B <= n ? B : n - j * B;
-            FO_CUDA(mlp_gather_norm(d_feat, idx + j * B, Bj, kMlpIn, norm, norm + kMlpIn, xb, st), "batch");
-            FO_CUDA(mlp_gather_norm(d_target, idx + j * B, Bj, kMlpOut, norm + 2 * kMlpIn,
-                                    norm + 2 * kMlpIn + kMlpOut, tb, st),
-                    "batch");
-            FO_CUDA(mlp_forward(mlp_params(ctx), xb, Bj, z1, a1, z2, a2, y, st), "network");
-            FO_CUDA(mlp_backward(mlp_params(ctx), xb, tb, Bj, z1, a1, z2, a2, y, dy, dz2, dz1, mlp_grad(ctx),
-                                 losses + step_i, st),
-                    "backward");
             ctx->mlp_step += 1;
-            FO_CUDA(mlp_adam(mlp_params(ctx), mlp_grad(ctx), mlp_m(ctx), mlp_v(ctx), P, lr, ctx->mlp_step, st),
-                    "adam");
+            MlpStep ms{};
+            ms.params = mlp_params(ctx);
+            ms.feat = d_feat;
+            ms.target = d_target;
+            ms.idx = idx + (size_t)j * B;
+            ms.norm = norm;
+            ms.B = (j + 1) * B <= n ? B : n - j * B;
+            ms.scratch = ctx->mlp_scratch;
+            ms.m = mlp_m(ctx);
+            ms.v = mlp_v(ctx);
+            ms.lr = lr;
+            ms.step = ctx->mlp_step;
+            ms.loss = losses + step_i;
+            FO_CUDA(mlp_step(ms, st), "training step");
         }
     }
     std::vector<float> hl(total_steps);

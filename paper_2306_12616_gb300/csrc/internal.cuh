@@ -434,15 +434,25 @@ inline MlpOffsets mlp_offsets() {
     o.total = o.b3 + kMlpOut;
     return o;
 }
-cudaError_t mlp_forward(const float* params, const float* x, int B, float* z1, float* a1, float* z2, float* a2,
-                        float* y, cudaStream_t s);
-// Loss of (y, t) into *loss, dL/dy into dy and every parameter gradient into grad.
-cudaError_t mlp_backward(const float* params, const float* x, const float* t, int B, const float* z1,
-                         const float* a1, const float* z2, const float* a2, const float* y, float* dy, float* dz2,
-                         float* dz1, float* grad, float* loss, cudaStream_t s);
-cudaError_t mlp_adam(float* p, const float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s);
-cudaError_t mlp_gather_norm(const float* src, const int* idx, int B, int C, const float* mean, const float* stdv,
-                            float* dst, cudaStream_t s);
+// Outputs y[B x 2] for inputs x[B x 68], standardised with norm (null: already standardised).
+cudaError_t mlp_forward(const float* params, const float* x, const float* norm, int B, float* y, cudaStream_t s);
+// One training step on B rows (row idx[b] of feat and target, or row b): loss, and either the
+// gradient of every parameter (grad) or one Adam step of params (grad null).
+struct MlpStep {
+    float* params;
+    const float *feat, *target;
+    const int* idx;
+    const float* norm;    // standardisation of feat and target (null: already standardised)
+    int B;
+    float* scratch;       // mlp_step_floats(B)
+    float* grad;
+    float *m, *v;         // Adam moments
+    float lr;
+    int step;             // Adam step, from 1
+    float* loss;
+};
+cudaError_t mlp_step(const MlpStep& st, cudaStream_t s);
+size_t mlp_step_floats(int B);
 cudaError_t mlp_col_stats(const float* X, int n, int C, float* mean, float* stdv, cudaStream_t s);
 cudaError_t launch_features(const Inst* in, const InstIO* io, int batch, int k, int rows_by_user, float* feat,
                             cudaStream_t s);

@@ -11,7 +11,11 @@
 //
 // Every reduction runs in a fixed order (one thread per output, sequential sums), so
 // training and inference are deterministic.
+#include <cooperative_groups.h>
+
 #include "internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace fo {
 namespace {
@@ -22,87 +26,343 @@ __device__ __forceinline__ float silu_grad_f(float z) {
     return s * (1.0f + z * (1.0f - s));
 }
 
-// out[b, o] = act(sum_i in[b, i] W[o, i] + bias[o]); z[b, o] = the pre-activation.
-__global__ void k_dense_fwd(const float* __restrict__ in, int B, int I, const float* __restrict__ W,
-                            const float* __restrict__ bias, int O, int act, float* __restrict__ z,
-                            float* __restrict__ out) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (o >= O || b >= B) return;
-    const float* x = in + (int64_t)b * I;
-    const float* w = W + (int64_t)o * I;
-    float s = bias[o];
-    for (int i = 0; i < I; ++i) s = fmaf(x[i], w[i], s);
-    if (z) z[(int64_t)b * O + o] = s;
-    out[(int64_t)b * O + o] = act ? silu_f(s) : s;
-}
+// ------------------------------------------------------------------ rows of a batch
+// Everything of a training step that is local to a row of the batch: gather and standardise, the
+// three layers, the loss gradient and the gradients of the pre-activations. A cluster of kCl CTAs
+// takes kRows rows; each CTA holds 256 / kCl hidden units of either layer: its rows of W1 and W2
+// and its columns of W2 (the backward pass) are copied to shared memory at the start, while the
+// first layer runs, and activations are exchanged through distributed shared memory (three
+// times). The weights' bytes bound it: 145 KB per CTA from L2, about 2300 clocks, as long as the
+// sums of a layer; one CTA per two rows would read all 580 KB. Every sum runs in the order of its
+// definition, one term after another in one thread.
+// One training step of 256 rows, with k_mlp_grad: 16.4 + 13.3 us in 2 launches, where 11 launches
+// took about 205 us (20000 rows, two epochs: 33.5 -> 5.3 ms).
+constexpr int kCl = 4;                          // CTAs per cluster
+constexpr int kRows = 8;                        // rows per cluster
+constexpr int kUnits = kMlpHidden / kCl;        // hidden units per CTA
+constexpr int kRowThreads = kUnits * (kRows / 2);   // a thread: one unit, two rows
+constexpr int kLd1 = kMlpIn;                    // shared strides: an odd number of 16-byte words, so that
+constexpr int kLd2 = kMlpHidden + 4;            // the rows of a warp's lanes start in different banks
+static_assert(kLd1 % 8 == 4 && kLd2 % 8 == 4, "strides");
 
-// dW[o, i] = sum_b dZ[b, o] A[b, i]; db[o] = sum_b dZ[b, o] (thread (o, I) does the bias).
-__global__ void k_dense_bwd_w(const float* __restrict__ dZ, const float* __restrict__ A, int B, int I, int O,
-                              float* __restrict__ dW, float* __restrict__ db) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y;
-    if (i > I || o >= O) return;
-    float s = 0.0f;
-    if (i < I) {
-        for (int b = 0; b < B; ++b) s = fmaf(dZ[(int64_t)b * O + o], A[(int64_t)b * I + i], s);
-        dW[(int64_t)o * I + i] = s;
-    } else {
-        for (int b = 0; b < B; ++b) s += dZ[(int64_t)b * O + o];
-        db[o] = s;
+struct RowSmem {
+    float w1[kUnits * kLd1];          // rows of W1
+    float w2r[kUnits * kLd2];         // rows of W2 (forward)
+    float w2c[kMlpHidden * kUnits];   // columns of W2 (backward)
+    float w3[kMlpOut * kMlpHidden];
+    float x[kRows * kMlpIn];
+    float a1[kRows * kMlpHidden];
+    float a2[kRows * kMlpHidden];
+    float dz2[kRows * kMlpHidden];
+    float y[kRows * kMlpOut], dy[kRows * kMlpOut];
+};
+
+struct RowArgs {
+    const float *params, *src, *tsrc;   // parameters; features and targets [. x 68], [. x 2]
+    const int* idx;                     // rows of src / tsrc (null: row b)
+    const float* norm;                  // standardisation (null: src and tsrc are standardised)
+    int B;
+    float *x, *t;                       // standardised rows [B x 68], [B x 2] (training)
+    float *a1, *a2, *dz1, *dz2;         // [B x 256]
+    float *y, *dy;                      // [B x 2]
+};
+
+template <bool TRAIN>
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp_rows(const RowArgs g) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    RowSmem& sm = *reinterpret_cast<RowSmem*>(raw);
+    cg::cluster_group cl = cg::this_cluster();
+    const int c = (int)cl.block_rank(), u0 = c * kUnits;
+    const int b0 = ((int)blockIdx.x / kCl) * kRows, tid = threadIdx.x;
+    const float* W1 = g.params;
+    const float* B1 = W1 + kMlpHidden * kMlpIn;
+    const float* W2 = B1 + kMlpHidden;
+    const float* B2 = W2 + kMlpHidden * kMlpHidden;
+    const float* W3 = B2 + kMlpHidden;
+    const float* B3 = W3 + kMlpOut * kMlpHidden;
+    // group 0: the rows and W1; group 1: W2's rows and W3; group 2: W2's columns
+    for (int q = tid; q < kUnits * (kMlpIn / 4); q += kRowThreads) {
+        const int o = q / (kMlpIn / 4), i = 4 * (q - o * (kMlpIn / 4));
+        cp_async16(&sm.w1[o * kLd1 + i], W1 + (u0 + o) * kMlpIn + i);
     }
-}
-
-// dZprev[b, i] = (sum_o dZ[b, o] W[o, i]) silu'(zprev[b, i]).
-__global__ void k_dense_bwd_x(const float* __restrict__ dZ, const float* __restrict__ W, int B, int I, int O,
-                              const float* __restrict__ zprev, float* __restrict__ dZprev) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (i >= I || b >= B) return;
-    float s = 0.0f;
-    for (int o = 0; o < O; ++o) s = fmaf(dZ[(int64_t)b * O + o], W[(int64_t)o * I + i], s);
-    dZprev[(int64_t)b * I + i] = s * silu_grad_f(zprev[(int64_t)b * I + i]);
-}
-
-// Weighted squared error L = (1/B) sum_b sum_j w_j (y - t)^2 and dL/dy; one block.
-__global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, int B, float w0, float w1,
-                      float* __restrict__ dy, float* __restrict__ loss) {
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int q = threadIdx.x; q < 2 * B; q += blockDim.x) {
-        const float w = (q & 1) ? w1 : w0;
-        const float d = y[q] - t[q];
-        dy[q] = 2.0f * w * d / (float)B;
-        s += (double)w * d * d;
+    cp_async_commit();
+    for (int q = tid; q < kUnits * (kMlpHidden / 4); q += kRowThreads) {
+        const int o = q / (kMlpHidden / 4), i = 4 * (q - o * (kMlpHidden / 4));
+        cp_async16(&sm.w2r[o * kLd2 + i], W2 + (u0 + o) * kMlpHidden + i);
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    for (int q = tid; q < kMlpOut * kMlpHidden; q += kRowThreads) sm.w3[q] = W3[q];
+    cp_async_commit();
+    if (TRAIN) {
+        for (int q = tid; q < kMlpHidden * (kUnits / 4); q += kRowThreads) {
+            const int o = q / (kUnits / 4), i = 4 * (q - o * (kUnits / 4));
+            cp_async16(&sm.w2c[o * kUnits + i], W2 + o * kMlpHidden + u0 + i);
+        }
+    }
+    cp_async_commit();
+    for (int q = tid; q < kRows * kMlpIn; q += kRowThreads) {
+        const int rr = q / kMlpIn, i = q - rr * kMlpIn, b = b0 + rr;
+        float v = 0.0f;
+        if (b < g.B) {
+            v = g.src[(int64_t)(g.idx ? g.idx[b] : b) * kMlpIn + i];
+            if (g.norm) v = (v - g.norm[i]) / g.norm[kMlpIn + i];
+            if (TRAIN && c == 0) g.x[(int64_t)b * kMlpIn + i] = v;
+        }
+        sm.x[q] = v;
+    }
+    cp_async_wait<2>();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += sh[w];
-        *loss = (float)(tot / B);
+    cl.sync();   // every CTA of the cluster runs before its shared memory is written
+    // this thread: hidden unit u0 + o of rows 2 rg, 2 rg + 1
+    const int o = tid % kUnits, rg = tid / kUnits, r0 = 2 * rg;
+    auto share = [&](float* dst, float v0, float v1) {   // into every CTA's copy
+#pragma unroll
+        for (int q = 0; q < kCl; ++q) {
+            float* d = cl.map_shared_rank(dst, q);
+            d[r0 * kMlpHidden + u0 + o] = v0;
+            d[(r0 + 1) * kMlpHidden + u0 + o] = v1;
+        }
+    };
+    auto keep = [&](float* dst, float v0, float v1) {     // [B x 256] in global memory
+        if (b0 + r0 < g.B) dst[(int64_t)(b0 + r0) * kMlpHidden + u0 + o] = v0;
+        if (b0 + r0 + 1 < g.B) dst[(int64_t)(b0 + r0 + 1) * kMlpHidden + u0 + o] = v1;
+    };
+    auto layer = [&](const float* w, const float* in, int n, float bias, float& s0, float& s1) {
+        s0 = s1 = bias;
+        const float *x0 = in + r0 * n, *x1 = x0 + n;
+#pragma unroll 4
+        for (int i = 0; i < n; i += 4) {
+            const float4 wv = *reinterpret_cast<const float4*>(w + i);
+            const float4 p = *reinterpret_cast<const float4*>(x0 + i), q = *reinterpret_cast<const float4*>(x1 + i);
+            s0 = fmaf(p.x, wv.x, s0);
+            s1 = fmaf(q.x, wv.x, s1);
+            s0 = fmaf(p.y, wv.y, s0);
+            s1 = fmaf(q.y, wv.y, s1);
+            s0 = fmaf(p.z, wv.z, s0);
+            s1 = fmaf(q.z, wv.z, s1);
+            s0 = fmaf(p.w, wv.w, s0);
+            s1 = fmaf(q.w, wv.w, s1);
+        }
+    };
+    float z10, z11, z20, z21;
+    layer(sm.w1 + o * kLd1, sm.x, kMlpIn, B1[u0 + o], z10, z11);
+    {
+        const float v0 = silu_f(z10), v1 = silu_f(z11);
+        share(sm.a1, v0, v1);
+        if (TRAIN) keep(g.a1, v0, v1);
+    }
+    cp_async_wait<1>();
+    cl.sync();
+    layer(sm.w2r + o * kLd2, sm.a1, kMlpHidden, B2[u0 + o], z20, z21);
+    {
+        const float v0 = silu_f(z20), v1 = silu_f(z21);
+        share(sm.a2, v0, v1);
+        if (TRAIN) keep(g.a2, v0, v1);
+    }
+    cp_async_wait<0>();
+    cl.sync();
+    if (tid < kRows * kMlpOut) {
+        // the outputs, in every CTA (the backward pass of each needs them)
+        const int rr = tid / kMlpOut, j = tid - rr * kMlpOut, b = b0 + rr;
+        float s = B3[j];
+        const float *w = sm.w3 + j * kMlpHidden, *a = sm.a2 + rr * kMlpHidden;
+#pragma unroll 8
+        for (int i = 0; i < kMlpHidden; ++i) s = fmaf(a[i], w[i], s);
+        if (b < g.B) {
+            if (c == 0) g.y[(int64_t)b * kMlpOut + j] = s;
+            if (TRAIN) {
+                float t = g.tsrc[(int64_t)(g.idx ? g.idx[b] : b) * kMlpOut + j];
+                if (g.norm) t = (t - g.norm[2 * kMlpIn + j]) / g.norm[2 * kMlpIn + kMlpOut + j];
+                const float wl = j ? kMlpLossW1 : kMlpLossW0;
+                const float d = s - t;
+                const float dv = 2.0f * wl * d / (float)g.B;
+                sm.dy[tid] = dv;
+                if (c == 0) {
+                    g.t[(int64_t)b * kMlpOut + j] = t;
+                    g.dy[(int64_t)b * kMlpOut + j] = dv;
+                }
+            }
+        } else if (TRAIN) {
+            sm.dy[tid] = 0.0f;
+        }
+    }
+    if (!TRAIN) return;   // (no CTA touches another's shared memory past the last cl.sync)
+    __syncthreads();
+    {
+        // dz2 = (sum_j dy_j W3[j, .]) silu'(z2)
+        float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+        for (int j = 0; j < kMlpOut; ++j) {
+            const float w = sm.w3[j * kMlpHidden + u0 + o];
+            s0 = fmaf(sm.dy[r0 * kMlpOut + j], w, s0);
+            s1 = fmaf(sm.dy[(r0 + 1) * kMlpOut + j], w, s1);
+        }
+        const float v0 = s0 * silu_grad_f(z20), v1 = s1 * silu_grad_f(z21);
+        share(sm.dz2, v0, v1);
+        keep(g.dz2, v0, v1);
+    }
+    cl.sync();
+    {
+        // dz1 = (sum_o dz2_o W2[o, .]) silu'(z1)
+        float s0 = 0.0f, s1 = 0.0f;
+        const float *p = sm.dz2 + r0 * kMlpHidden, *q = p + kMlpHidden;
+#pragma unroll 4
+        for (int k = 0; k < kMlpHidden; k += 4) {
+            const float4 d0 = *reinterpret_cast<const float4*>(p + k), d1 = *reinterpret_cast<const float4*>(q + k);
+            const float* w = sm.w2c + k * kUnits + o;
+            s0 = fmaf(d0.x, w[0], s0);
+            s1 = fmaf(d1.x, w[0], s1);
+            s0 = fmaf(d0.y, w[kUnits], s0);
+            s1 = fmaf(d1.y, w[kUnits], s1);
+            s0 = fmaf(d0.z, w[2 * kUnits], s0);
+            s1 = fmaf(d1.z, w[2 * kUnits], s1);
+            s0 = fmaf(d0.w, w[3 * kUnits], s0);
+            s1 = fmaf(d1.w, w[3 * kUnits], s1);
+        }
+        keep(g.dz1, s0 * silu_grad_f(z10), s1 * silu_grad_f(z11));
     }
 }
 
-// Adam (Kingma and Ba) with bias-corrected moments; step counts from 1.
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int n, float lr, float b1, float b2, float eps, int step) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const float mq = b1 * m[q] + (1.0f - b1) * g[q];
-    const float vq = b2 * v[q] + (1.0f - b2) * g[q] * g[q];
-    m[q] = mq;
-    v[q] = vq;
-    const float mh = mq / (1.0f - powf(b1, (float)step));
-    const float vh = vq / (1.0f - powf(b2, (float)step));
-    p[q] -= lr * mh / (sqrtf(vh) + eps);
-}
+// ------------------------------------------------------------------ weight gradients, Adam, loss
+// dW[o, i] = sum_b dZ[b, o] A[b, i] (one thread per parameter group, b in order), db[o] = sum_b
+// dZ[b, o] as the column i = I with A = 1, of all three layers in one launch, then either the
+// gradient itself or one Adam step of the parameter (Kingma and Ba, bias-corrected, step from 1);
+// one more block adds the loss. A block: kGo outputs x kGi inputs, 128 threads of 1 x 4 parameters;
+// 16 x 32 tiles give 202 blocks for the 152 SMs. Latency bounds it, so dZ and A are requested whole
+// (up to kGb rows) by asynchronous copies before any sum starts (13.3 us; four staged passes took 17).
+constexpr int kGo = 16, kGi = 32, kGb = 256;
+constexpr int kGradSmem = kGb * (kGo + kGi) * 4;
+constexpr int kTilesI1 = (kMlpIn + 1 + kGi - 1) / kGi, kTilesI2 = (kMlpHidden + 1 + kGi - 1) / kGi;
+constexpr int kTilesO = kMlpHidden / kGo;
+constexpr int kGradBlocks = kTilesO * kTilesI1 + kTilesO * kTilesI2 + kTilesI2 + 1;
 
-// dst[r, :] = (src[idx[r], :] - mean) / std
-__global__ void k_gather_norm(const float* __restrict__ src, const int* __restrict__ idx, int B, int C,
-                              const float* __restrict__ mean, const float* __restrict__ stdv, float* __restrict__ dst) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
-    if (c >= C || r >= B) return;
-    const int s = idx ? idx[r] : r;
-    dst[(int64_t)r * C + c] = (src[(int64_t)s * C + c] - mean[c]) / stdv[c];
+struct GradArgs {
+    const float *x, *a1, *a2, *dz1, *dz2, *dy, *y, *t;
+    int B;
+    float* grad;          // gradient out (null: Adam)
+    float *p, *m, *v;     // Adam: parameters and moments
+    float lr;
+    int step;
+    float* loss;
+};
+
+__global__ void __launch_bounds__(128) k_mlp_grad(const GradArgs g) {
+    extern __shared__ __align__(16) float gsm[];
+    float (*sz)[kGo] = reinterpret_cast<float (*)[kGo]>(gsm);
+    float (*sa)[kGi] = reinterpret_cast<float (*)[kGi]>(gsm + kGb * kGo);
+    __shared__ float s_corr[2];
+    const int tid = threadIdx.x;
+    int blk = blockIdx.x;
+    if (blk == kGradBlocks - 1) {
+        // L = (1/B) sum_b sum_j w_j (y - t)^2: 256 strided float64 sums (two per thread here), a
+        // shuffle tree per 32 of them, their eight results in order
+        __shared__ double sh[8];
+        for (int half = 0; half < 2; ++half) {
+            double s = 0.0;
+            for (int q = tid + 128 * half; q < 2 * g.B; q += 256) {
+                const float w = (q & 1) ? kMlpLossW1 : kMlpLossW0;
+                const float d = g.y[q] - g.t[q];
+                s += (double)w * d * d;
+            }
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((tid & 31) == 0) sh[4 * half + (tid >> 5)] = s;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            double tot = 0.0;
+            for (int w = 0; w < 8; ++w) tot += sh[w];
+            *g.loss = (float)(tot / g.B);
+        }
+        return;
+    }
+    // layer, output tile, input tile; parameters W (O x I) at off, then the O biases
+    const float *dz, *A;
+    int O, I, off, ot, it;
+    if (blk < kTilesO * kTilesI2) {
+        dz = g.dz2;
+        A = g.a1;
+        O = kMlpHidden;
+        I = kMlpHidden;
+        off = kMlpHidden * kMlpIn + kMlpHidden;
+        ot = blk / kTilesI2;
+        it = blk - ot * kTilesI2;
+    } else if ((blk -= kTilesO * kTilesI2) < kTilesO * kTilesI1) {
+        dz = g.dz1;
+        A = g.x;
+        O = kMlpHidden;
+        I = kMlpIn;
+        off = 0;
+        ot = blk / kTilesI1;
+        it = blk - ot * kTilesI1;
+    } else {
+        blk -= kTilesO * kTilesI1;
+        dz = g.dy;
+        A = g.a2;
+        O = kMlpOut;
+        I = kMlpHidden;
+        off = kMlpHidden * kMlpIn + kMlpHidden + kMlpHidden * kMlpHidden + kMlpHidden;
+        ot = 0;
+        it = blk;
+    }
+    const int o0 = ot * kGo, i0 = it * kGi;
+    if (!g.grad && tid == 0) {
+        s_corr[0] = 1.0f - powf(0.9f, (float)g.step);
+        s_corr[1] = 1.0f - powf(0.999f, (float)g.step);
+    }
+    const int o = tid >> 3, i4 = (tid & 7) * 4;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int b0 = 0; b0 < g.B; b0 += kGb) {
+        const int nb = g.B - b0 < kGb ? g.B - b0 : kGb;
+        __syncthreads();
+        if (O % 4 == 0) {
+            for (int q = tid; q < nb * (kGo / 4); q += 128) {
+                const int b = q / (kGo / 4), oo = 4 * (q % (kGo / 4));
+                cp_async16(&sz[b][oo], dz + (int64_t)(b0 + b) * O + o0 + oo);
+            }
+        } else {
+            for (int q = tid; q < nb * kGo; q += 128) {
+                const int b = q / kGo, oo = q % kGo;
+                sz[b][oo] = o0 + oo < O ? dz[(int64_t)(b0 + b) * O + o0 + oo] : 0.0f;
+            }
+        }
+        for (int q = tid; q < nb * (kGi / 4); q += 128) {
+            const int b = q / (kGi / 4), ii = 4 * (q % (kGi / 4));
+            // (I is a multiple of 4: a group of four columns is inside the inputs, or starts at the
+            // bias column, or lies past it)
+            if (i0 + ii < I) cp_async16(&sa[b][ii], A + (int64_t)(b0 + b) * I + i0 + ii);
+            else *reinterpret_cast<float4*>(&sa[b][ii]) = make_float4(i0 + ii == I ? 1.0f : 0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+#pragma unroll 8
+        for (int b = 0; b < nb; ++b) {
+            const float z = sz[b][o];
+            const float4 a = *reinterpret_cast<const float4*>(&sa[b][i4]);
+            s[0] = fmaf(z, a.x, s[0]);
+            s[1] = fmaf(z, a.y, s[1]);
+            s[2] = fmaf(z, a.z, s[2]);
+            s[3] = fmaf(z, a.w, s[3]);
+        }
+    }
+    if (o0 + o >= O) return;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = i0 + i4 + u;
+        if (i > I) break;
+        const int q = i < I ? off + (o0 + o) * I + i : off + O * I + o0 + o;
+        if (g.grad) {
+            g.grad[q] = s[u];
+        } else {
+            const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+            const float mq = b1 * g.m[q] + (1.0f - b1) * s[u];
+            const float vq = b2 * g.v[q] + (1.0f - b2) * s[u] * s[u];
+            g.m[q] = mq;
+            g.v[q] = vq;
+            const float mh = mq / s_corr[0];
+            const float vh = vq / s_corr[1];
+            g.p[q] -= g.lr * mh / (sqrtf(vh) + eps);
+        }
+    }
 }
 
 // Column mean and standard deviation (float64 sums in row order); std floored at 1e-6 of
@@ -264,48 +524,73 @@ __global__ void k_learned_check(const Inst* __restrict__ insts, const InstIO* __
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-cudaError_t mlp_forward(const float* params, const float* x, int B, float* z1, float* a1, float* z2, float* a2,
-                        float* y, cudaStream_t s) {
+namespace {
+template <bool TRAIN>
+cudaError_t launch_rows(const RowArgs& a, cudaStream_t s) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_mlp_rows<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowSmem));
+    if (e != cudaSuccess) return e;
+    k_mlp_rows<TRAIN><<<(unsigned)((a.B + kRows - 1) / kRows * kCl), kRowThreads, sizeof(RowSmem), s>>>(a);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t mlp_forward(const float* params, const float* x, const float* norm, int B, float* y, cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
-    const MlpOffsets o = mlp_offsets();
-    k_dense_fwd<<<dim3((kMlpHidden + 127) / 128, B), 128, 0, s>>>(x, B, kMlpIn, params + o.W1, params + o.b1,
-                                                                  kMlpHidden, 1, z1, a1);
-    k_dense_fwd<<<dim3((kMlpHidden + 127) / 128, B), 128, 0, s>>>(a1, B, kMlpHidden, params + o.W2, params + o.b2,
-                                                                  kMlpHidden, 1, z2, a2);
-    k_dense_fwd<<<dim3(1, B), 32, 0, s>>>(a2, B, kMlpHidden, params + o.W3, params + o.b3, kMlpOut, 0, nullptr, y);
-    return cudaGetLastError();
+    RowArgs a{};
+    a.params = params;
+    a.src = x;
+    a.norm = norm;
+    a.B = B;
+    a.y = y;
+    return launch_rows<false>(a, s);
 }
 
-cudaError_t mlp_backward(const float* params, const float* x, const float* t, int B, const float* z1,
-                         const float* a1, const float* z2, const float* a2, const float* y, float* dy, float* dz2,
-                         float* dz1, float* grad, float* loss, cudaStream_t s) {
-    const MlpOffsets o = mlp_offsets();
-    k_mse<<<1, 256, 0, s>>>(y, t, B, kMlpLossW0, kMlpLossW1, dy, loss);
-    k_dense_bwd_w<<<dim3((kMlpHidden + 1 + 127) / 128, kMlpOut), 128, 0, s>>>(dy, a2, B, kMlpHidden, kMlpOut,
-                                                                              grad + o.W3, grad + o.b3);
-    k_dense_bwd_x<<<dim3((kMlpHidden + 127) / 128, B), 128, 0, s>>>(dy, params + o.W3, B, kMlpHidden, kMlpOut,
-                                                                    z2, dz2);
-    k_dense_bwd_w<<<dim3((kMlpHidden + 1 + 127) / 128, kMlpHidden), 128, 0, s>>>(dz2, a1, B, kMlpHidden,
-                                                                                 kMlpHidden, grad + o.W2,
-                                                                                 grad + o.b2);
-    k_dense_bwd_x<<<dim3((kMlpHidden + 127) / 128, B), 128, 0, s>>>(dz2, params + o.W2, B, kMlpHidden,
-                                                                    kMlpHidden, z1, dz1);
-    k_dense_bwd_w<<<dim3((kMlpIn + 1 + 127) / 128, kMlpHidden), 128, 0, s>>>(dz1, x, B, kMlpIn, kMlpHidden,
-                                                                             grad + o.W1, grad + o.b1);
+cudaError_t mlp_step(const MlpStep& st, cudaStream_t s) {
+    if (st.B <= 0) return cudaSuccess;
+    const size_t B = (size_t)st.B;
+    RowArgs a{};
+    a.params = st.params;
+    a.src = st.feat;
+    a.tsrc = st.target;
+    a.idx = st.idx;
+    a.norm = st.norm;
+    a.B = st.B;
+    float* w = st.scratch;
+    auto take = [&](size_t n) { float* r = w; w += (n + 3) & ~size_t(3); return r; };   // 16-byte aligned
+    a.x = take(B * kMlpIn);
+    a.t = take(B * kMlpOut);
+    a.a1 = take(B * kMlpHidden);
+    a.a2 = take(B * kMlpHidden);
+    a.dz1 = take(B * kMlpHidden);
+    a.dz2 = take(B * kMlpHidden);
+    a.y = take(B * kMlpOut);
+    a.dy = take(B * kMlpOut);
+    const cudaError_t e = launch_rows<true>(a, s);
+    if (e != cudaSuccess) return e;
+    GradArgs g{};
+    g.x = a.x;
+    g.a1 = a.a1;
+    g.a2 = a.a2;
+    g.dz1 = a.dz1;
+    g.dz2 = a.dz2;
+    g.dy = a.dy;
+    g.y = a.y;
+    g.t = a.t;
+    g.B = st.B;
+    g.grad = st.grad;
+    g.p = st.params;
+    g.m = st.m;
+    g.v = st.v;
+    g.lr = st.lr;
+    g.step = st.step;
+    g.loss = st.loss;
+    const cudaError_t eg = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem);
+    if (eg != cudaSuccess) return eg;
+    k_mlp_grad<<<kGradBlocks, 128, kGradSmem, s>>>(g);
     return cudaGetLastError();
 }
-
-cudaError_t mlp_adam(float* p, const float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s) {
-    k_adam<<<(n + 255) / 256, 256, 0, s>>>(p, g, m, v, n, lr, 0.9f, 0.999f, 1e-8f, step);
-    return cudaGetLastError();
-}
-
-cudaError_t mlp_gather_norm(const float* src, const int* idx, int B, int C, const float* mean, const float* stdv,
-                            float* dst, cudaStream_t s) {
-    if (B <= 0) return cudaSuccess;
-    k_gather_norm<<<dim3((C + 127) / 128, B), 128, 0, s>>>(src, idx, B, C, mean, stdv, dst);
-    return cudaGetLastError();
-}
+size_t mlp_step_floats(int B) { return (size_t)B * (kMlpIn + 3 * kMlpOut + 4 * kMlpHidden) + 3 * 4; }
 
 cudaError_t mlp_col_stats(const float* X, int n, int C, float* mean, float* stdv, cudaStream_t s) {
     k_col_stats<<<C, 256, 0, s>>>(X, n, C, mean, stdv);
