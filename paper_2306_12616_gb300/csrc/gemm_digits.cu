@@ -102,19 +102,6 @@ __host__ __device__ constexpr int acc_order(int q, int l, int gs) {
     return q;
 }
 
-// One MMA of the elected lane (lead != 0) of a converged warp, its descriptors given by their low
-// words (address and leading offset) and a common high word. The predicate is part of the
-// instruction instead of a branch around it, so that the warp's control flow stays uniform and
-// the descriptors in uniform registers.
-__device__ __forceinline__ void umma_lo(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t acc,
-                                        uint32_t lead) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 e, %6, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}\n" ::"r"(tmem_d),
-        "r"(alo), "r"(blo), "r"(hi), "r"(kIdesc), "r"(acc), "r"(lead));
-}
 // The O + 1 digit pairs of order O for one k16 block.
 template <int O>
 __device__ __forceinline__ void issue_order(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, bool fresh,
@@ -122,8 +109,9 @@ __device__ __forceinline__ void issue_order(uint32_t tmem_d, uint32_t alo, uint3
 #pragma unroll
     for (int i = 0; i <= O; ++i) {
         const int j = O - i;
-        umma_lo(tmem_d, alo + (uint32_t)((i >> 2) * (kBoxBytes >> 4) + (i & 3) * 2),
-                blo + (uint32_t)((j >> 2) * (kBoxBytes >> 4) + (j & 3) * 2), hi, i > 0 ? 1u : (fresh ? 0u : 1u), lead);
+        umma_lead(tmem_d, alo + (uint32_t)((i >> 2) * (kBoxBytes >> 4) + (i & 3) * 2), hi,
+                  blo + (uint32_t)((j >> 2) * (kBoxBytes >> 4) + (j & 3) * 2), hi, kIdesc,
+                  i > 0 ? 1u : (fresh ? 0u : 1u), lead);
     }
 }
 

@@ -288,7 +288,8 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     const bool ub = sym == 2;   // upper-block storage: lower operand blocks read transposed
     const int ib = in.in_bucket;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the warp index through a shuffle: a role's branch is then known to be uniform
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int tm = np / kBM, tn = (np + TBN - 1) / TBN;
     int I, J;
     tile_of(gtile - __ldg(pre + inst), tm, tn, TBN, sym, I, J);
@@ -446,74 +447,81 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer: one k-block per accumulator, corrections first.
-            // The loop is instantiated once per plane storage, so the K-major one carries no
-            // trace of the MN-major layouts (a runtime layout branch in it cost 5%).
-            // Descriptors: the address field (bits 0-13, address / 16) of a stage's operand is
-            // the ring base's plus a compile-time offset, so each MMA's descriptor is one add.
-            const uint64_t d_k = sdesc_sw64(smem_u32(smem)), d_mn = sdesc_mn128(smem_u32(smem));
-            auto issue = [&](auto ub_tag) {
-                constexpr bool U = decltype(ub_tag)::value;
-                for (int kb = 0; kb < nk; ++kb) {
-                    const int s = kb % S, buf = kb & 1;
-                    // operand layouts of this k-block (see the producer): K-major tiles advance
-                    // 32 bytes per k16 slice, MN-major tiles 16 rows (2 KB)
-                    const int KB = kb * kBK / kBM;
-                    const bool a_mn = U && KB < m0 / kBM;
-                    const bool b0_mn = U && KB < n0 / kBM;
-                    const bool b1_mn = U && KB < n0 / kBM + 1;
-                    const uint64_t so = (uint64_t)s * (uint64_t)(Cfg::kStageBytes >> 4);
-                    auto adesc = [&](int p, int kk) {
-                        return a_mn ? d_mn + so + (uint64_t)((p * kBoxBytes + kk * kMnKStep) >> 4)
-                                    : d_k + so + (uint64_t)((p * kBoxBytes + kk * 32) >> 4);
-                    };
-                    auto bdesc = [&](int p, int kk, int j, bool mn) {
-                        const int off = PA * kBoxBytes + (p * Cfg::kBBoxes + j) * kBoxBytes;
-                        return mn ? d_mn + so + (uint64_t)((off + kk * kMnKStep) >> 4)
-                                  : d_k + so + (uint64_t)((off + kk * 32) >> 4);
-                    };
-                    if (kb >= 2) {
-                        if (!mbar_wait(&seg_empty[buf], ((kb >> 1) - 1) & 1, kWaitNs, vabort)) {
-                            atomicExch(&abort_flag, 1);
-                            atomicExch(err_flag, 1);
-                            break;
-                        }
-                    }
-                    if (!mbar_wait(&full[s], (kb / S) & 1, kWaitNs, vabort)) {
+        // ---------------- MMA issuer: one k-block per accumulator, corrections first. The whole warp
+        // keeps the loop, one elected lane issues (umma_lead). The loop is instantiated once per
+        // plane storage, so the K-major one carries no trace of the MN-major layouts (a runtime
+        // layout branch in it cost 5%). Descriptors: the address field (bits 0-13, address / 16) of a
+        // stage's operand is the ring base's plus a compile-time offset.
+        const uint32_t lead = elect_one() ? 1u : 0u;
+        const uint64_t d_k = sdesc_sw64(smem_u32(smem)), d_mn = sdesc_mn128(smem_u32(smem));
+        const uint32_t k_lo = (uint32_t)d_k, k_hi = (uint32_t)(d_k >> 32);
+        const uint32_t mn_lo = (uint32_t)d_mn, mn_hi = (uint32_t)(d_mn >> 32);
+        auto issue = [&](auto ub_tag) {
+            constexpr bool U = decltype(ub_tag)::value;
+            int s = 0;
+            uint32_t ph = 0;   // ring slot of this k-block and the parity of its use
+            for (int kb = 0; kb < nk; ++kb) {
+                const int buf = kb & 1;
+                // operand layouts of this k-block (see the producer): K-major tiles advance
+                // 32 bytes per k16 slice, MN-major tiles 16 rows (2 KB)
+                const int KB = kb * kBK / kBM;
+                const bool a_mn = U && KB < m0 / kBM;
+                const bool b0_mn = U && KB < n0 / kBM;
+                const bool b1_mn = U && KB < n0 / kBM + 1;
+                const uint32_t so = (uint32_t)(s * (Cfg::kStageBytes >> 4));
+                const uint32_t ahi = a_mn ? mn_hi : k_hi;
+                auto alo = [&](int p, int kk) {
+                    return a_mn ? mn_lo + so + (uint32_t)((p * kBoxBytes + kk * kMnKStep) >> 4)
+                                : k_lo + so + (uint32_t)((p * kBoxBytes + kk * 32) >> 4);
+                };
+                auto blo = [&](int p, int kk, int j, bool mn) {
+                    const int off = PA * kBoxBytes + (p * Cfg::kBBoxes + j) * kBoxBytes;
+                    return mn ? mn_lo + so + (uint32_t)((off + kk * kMnKStep) >> 4)
+                              : k_lo + so + (uint32_t)((off + kk * 32) >> 4);
+                };
+                bool go = true;
+                if (kb >= 2) go = mbar_wait_warp(&seg_empty[buf], ((kb >> 1) - 1) & 1, kWaitNs, vabort);
+                if (go) go = mbar_wait_warp(&full[s], ph, kWaitNs, vabort);
+                if (!go) {
+                    if (lead) {
                         atomicExch(&abort_flag, 1);
                         atomicExch(err_flag, 1);
-                        break;
                     }
-                    fence_after();
-                    const uint32_t d = tmem + buf * TBN;
-                    // the two 128-column halves of B may differ in layout (the k-block of the
-                    // diagonal block of the first half): one MMA per half when they do
-                    const int halves = (!U || nbox == 1 || tile_k <= kBM || b0_mn == b1_mn) ? 1 : 2;
-                    for (int j = 0; j < halves; ++j) {
-                        const bool mn = j ? b1_mn : b0_mn;
-                        const uint32_t id = (halves == 1 ? idesc : idesc_f16(j ? tile_k - kBM : kBM, F16)) |
-                                            (a_mn ? kIdescMnA : 0u) | (mn ? kIdescMnB : 0u);
-#pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk) {
-#pragma unroll
-                            for (int pr = 1; pr < NPROD; ++pr)
-                                umma_f16(d + j * kBM, adesc(prod_a(pr), kk), bdesc(prod_b(pr), kk, j, mn), id,
-                                         !(kk == 0 && pr == 1));
-                        }
-#pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk)
-                            umma_f16(d + j * kBM, adesc(0, kk), bdesc(0, kk, j, mn), id, (NPROD > 1) || kk > 0);
-                    }
-                    umma_commit(&empty[s]);
-                    umma_commit(&seg_full[buf]);
+                    break;
                 }
-            };
-            if (ub) issue(std::true_type{});
-            else issue(std::false_type{});
-            // arrives once every issued MMA has completed (also after an abort)
-            umma_commit(acc_full);
-        }
+                fence_after();
+                const uint32_t d = tmem + buf * TBN;
+                // the two 128-column halves of B may differ in layout (the k-block of the
+                // diagonal block of the first half): one MMA per half when they do
+                const int halves = (!U || nbox == 1 || tile_k <= kBM || b0_mn == b1_mn) ? 1 : 2;
+                for (int j = 0; j < halves; ++j) {
+                    const bool mn = j ? b1_mn : b0_mn;
+                    const uint32_t bhi = mn ? mn_hi : k_hi;
+                    const uint32_t id = (halves == 1 ? idesc : idesc_f16(j ? tile_k - kBM : kBM, F16)) |
+                                        (a_mn ? kIdescMnA : 0u) | (mn ? kIdescMnB : 0u);
+#pragma unroll
+                    for (int kk = 0; kk < kBK / 16; ++kk) {
+#pragma unroll
+                        for (int pr = 1; pr < NPROD; ++pr)
+                            umma_lead(d + j * kBM, alo(prod_a(pr), kk), ahi, blo(prod_b(pr), kk, j, mn), bhi, id,
+                                      !(kk == 0 && pr == 1), lead);
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < kBK / 16; ++kk)
+                        umma_lead(d + j * kBM, alo(0, kk), ahi, blo(0, kk, j, mn), bhi, id, (NPROD > 1) || kk > 0,
+                                  lead);
+                }
+                umma_commit_if(&empty[s], lead);
+                umma_commit_if(&seg_full[buf], lead);
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+        };
+        if (ub) issue(std::true_type{});
+        else issue(std::false_type{});
+        umma_commit_if(acc_full, lead);   // arrives once every issued MMA has completed (also after an abort)
         __syncwarp();
     } else {
         // ---------------- drain warps: add every finished k-block to registers

@@ -56,6 +56,20 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
             smem_u32(bar))
         : "memory");
 }
+// One MMA of the elected lane (lead != 0) of a converged warp, its descriptors given as low words
+// (address and leading offset) and high words. The lane's predicate is part of the instruction
+// instead of a branch around it: the warp's control flow stays uniform and the descriptors in
+// uniform registers, which a single thread's branch denies them. Measured on 128-wide MMAs issued
+// in groups of 10 to 26: 146 to 209 clocks per MMA from one thread, 72 to 79 this way (hardware 64).
+__device__ __forceinline__ void umma_lead(uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                          uint32_t idesc, uint32_t accumulate, uint32_t lead) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 e, %7, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n" ::"r"(tmem_d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(lead));
+}
 // The commit of one lane (lead != 0) of a converged warp, without a branch.
 __device__ __forceinline__ void umma_commit_if(uint64_t* bar, uint32_t lead) {
     asm volatile(
