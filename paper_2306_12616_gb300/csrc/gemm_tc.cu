@@ -198,6 +198,15 @@ __device__ __forceinline__ void split3x2(float x0, float x1, bool f16, float psc
     }
 }
 
+// 16-byte word of the result tile that holds columns 4 c4 .. 4 c4 + 3 of row r: rows of TBN / 4
+// words, the low three bits of c4 exclusive-or'ed with a function of the row that takes eight values
+// over eight consecutive rows (the accumulators' writes), over every fourth row (the mirrored
+// reads) and is constant along a row (the row pass), so that none of them has bank conflicts.
+template <int TBN>
+__device__ __forceinline__ int slot_word(int r, int c4) {
+    return r * (TBN / 4) + (c4 ^ ((r & 7) ^ ((r >> 2) & 7)));
+}
+
 // Tile decode of one instance. Symmetric mode: the tiles of the 128-row block I that hold
 // an element with col >= row, i.e. column tiles J >= (128 I) / TBN, enumerated row by row.
 __device__ __forceinline__ void tile_of(int t, int tm, int tn, int tbn, int sym, int& I, int& J) {
@@ -590,15 +599,27 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     // is idle (every TMA load was consumed, every MMA completed), so it holds the 128 x TBN
     // float32 result tile; all global traffic below is coalesced across the warp.
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // Slot products (all but the one or two that write the caller's P or its trace partials) use
+    // 16-byte words with a swizzle (slot_word), the others rows of TBN + 1 floats.
     constexpr int LD = TBN + 1;
     float* tile = reinterpret_cast<float*>(smem);
+    const bool to_slot = !st.out64 && !st.part;
     {
         const int q = warp & 3, grp = (warp - 2) >> 2;
         const int rl = q * 32 + lane;
+        if (to_slot) {
+            float4* t4 = reinterpret_cast<float4*>(smem);
 #pragma unroll
-        for (int c = 0; c < NC / 2; ++c) {
-            tile[rl * LD + grp * NC + 2 * c] = st.alpha * sum[c].x;
-            tile[rl * LD + grp * NC + 2 * c + 1] = st.alpha * sum[c].y;
+            for (int c = 0; c < NC / 4; ++c)
+                t4[slot_word<TBN>(rl, grp * (NC / 4) + c)] =
+                    make_float4(st.alpha * sum[2 * c].x, st.alpha * sum[2 * c].y, st.alpha * sum[2 * c + 1].x,
+                                st.alpha * sum[2 * c + 1].y);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC / 2; ++c) {
+                tile[rl * LD + grp * NC + 2 * c] = st.alpha * sum[c].x;
+                tile[rl * LD + grp * NC + 2 * c + 1] = st.alpha * sum[c].y;
+            }
         }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * DW) : "memory");
@@ -687,11 +708,118 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
         }
     };
 
-    // The passes are instantiated twice: the products that write the caller's float64 P (with
-    // their trace partials) and all others, whose loops then carry none of that code (a shared
-    // loop with run-time checks made every product ~13 % slower).
-    auto passes = [&](auto f64_tag) {
-    constexpr bool F64 = decltype(f64_tag)::value;
+    // ---------------- slot products. A thread works on four neighbouring entries: one 16-byte load
+    // of C and of D, one 16-byte store of the master and one 8-byte store per plane, a warp on 128
+    // columns of one row. Instructions and latency bounded the pass when a thread took pairs of
+    // entries with per-entry predicates (clocks of a 128-wide tile at N = 1000: row pass 14700, now
+    // 6700; mirrored pass 8500, now 3800; of a 256-wide tile at N = 5000: 19700 and 12000, now 12400
+    // and 7300, beside 248000 of the products); now the stores' bytes bound it (256 KB per 128 x 128
+    // tile with full plane storage).
+    if (to_slot) {
+        float4* t4 = reinterpret_cast<float4*>(smem);
+        const bool master_low = st.lower_master != 0;
+        auto store4 = [&](int64_t o, float4 v, bool master) {
+            if (!FO_CHK(st.dbg, o >= 0 && o + 4 <= ld * ld && (o & 3) == 0, 112, o / ld, o % ld)) return;
+            if (master) *reinterpret_cast<float4*>(out_x + o) = v;
+            if (planes > 0) {
+                uint32_t a0, a1, a2, b0, b1, b2;
+                split3x2(v.x, v.y, F16, st.plane_scale, a0, a1, a2);
+                split3x2(v.z, v.w, F16, st.plane_scale, b0, b1, b2);
+                uint16_t* pl = out_p + o;
+                *reinterpret_cast<uint2*>(pl) = make_uint2(a0, b0);
+                if (PA > 1 && planes > 1) *reinterpret_cast<uint2*>(pl + pstride) = make_uint2(a1, b1);
+                if (PA > 2 && planes > 2) *reinterpret_cast<uint2*>(pl + 2 * pstride) = make_uint2(a2, b2);
+            }
+        };
+        // the tile's block on the diagonal (its first one), and whether the others are mirrored
+        const bool has_diag = sym && n0 == m0;
+        const bool mirror = sym && !(ub && !master_low);
+        // row pass: beta C + D + shift; the result stays in the tile, for the mirrored pass, and
+        // off the diagonal block goes to the slot. The loads of G iterations are issued together.
+        // (D may be the output slot itself, R_l -> b_l: each entry is read before it is written, by
+        // the same thread or, in the diagonal block, before the barrier; left of the diagonal C and
+        // D hold stale words there, whose results are never used.)
+        constexpr int RPW = kBM / DW, NB = TBN / kBM, NIT = RPW * NB;
+        constexpr int G = (DW == 16 || MINB == 2) ? 4 : 8;
+        static_assert(NIT % G == 0, "row-pass groups");
+#pragma unroll 1
+        for (int q0 = 0; q0 < NIT; q0 += G) {
+            float4 cv[G], dv[G];
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                const int q = q0 + u, r = ew * RPW + q / NB, b = q % NB;
+                const int64_t o = ((int64_t)m0 + r) * ld + n0 + b * kBM + 4 * lane;
+                cv[u] = dv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (b < nbox) {
+                    // within a chain launch other SMs wrote C and D during this launch: L2 loads
+                    if (Cm) cv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(Cm + o))
+                                          : *reinterpret_cast<const float4*>(Cm + o);
+                    if (Dm) dv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(Dm + o))
+                                          : *reinterpret_cast<const float4*>(Dm + o);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                const int q = q0 + u, r = ew * RPW + q / NB, b = q % NB;
+                if (b >= nbox) continue;   // past the matrix edge or the narrowed diagonal tile
+                float4* tw = t4 + slot_word<TBN>(r, b * (kBM / 4) + lane);
+                float4 v = *tw;
+                if (Cm) {
+                    v.x = fmaf(st.beta, cv[u].x, v.x);
+                    v.y = fmaf(st.beta, cv[u].y, v.y);
+                    v.z = fmaf(st.beta, cv[u].z, v.z);
+                    v.w = fmaf(st.beta, cv[u].w, v.w);
+                }
+                if (Dm) {
+                    v.x += dv[u].x;
+                    v.y += dv[u].y;
+                    v.z += dv[u].z;
+                    v.w += dv[u].w;
+                }
+                const int64_t grow = (int64_t)m0 + r, gcol = (int64_t)n0 + b * kBM + 4 * lane;
+                if (grow < n_real) {
+                    if (gcol == grow) v.x += st.shift;
+                    if (gcol + 1 == grow) v.y += st.shift;
+                    if (gcol + 2 == grow) v.z += st.shift;
+                    if (gcol + 3 == grow) v.w += st.shift;
+                }
+                const bool dblk = has_diag && b == 0;
+                if (dblk || mirror) *tw = v;
+                if (!dblk) store4(grow * ld + gcol, v, true);
+            }
+        }
+        if (sym) {
+            if (has_diag || mirror) asm volatile("bar.sync 1, %0;" ::"n"(32 * DW) : "memory");
+            if (has_diag) {
+                // the diagonal block whole, each entry left of the diagonal from its mirror
+#pragma unroll 2
+                for (int rr = 0; rr < RPW; ++rr) {
+                    const int r = ew * RPW + rr, c = 4 * lane;
+                    float4 v = t4[slot_word<TBN>(r, lane)];
+                    auto low = [&](int e) { return tile[4 * slot_word<TBN>(c + e, r >> 2) + (r & 3)]; };
+                    if (c < r) v.x = low(0);
+                    if (c + 1 < r) v.y = low(1);
+                    if (c + 2 < r) v.z = low(2);
+                    if (c + 3 < r) v.w = low(3);
+                    store4(((int64_t)m0 + r) * ld + n0 + c, v, true);
+                }
+            }
+            if (mirror) {
+                // four output rows n0 + c .. + 3 at a time: lanes on four neighbouring tile rows each
+                for (int g4 = ew + (has_diag ? kBM / 4 : 0); g4 < nbox * (kBM / 4); g4 += DW) {
+                    float4 a[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) a[i] = t4[slot_word<TBN>(4 * lane + i, g4)];
+                    const int64_t o = ((int64_t)n0 + 4 * g4) * ld + m0 + 4 * lane;
+                    store4(o, make_float4(a[0].x, a[1].x, a[2].x, a[3].x), master_low);
+                    store4(o + ld, make_float4(a[0].y, a[1].y, a[2].y, a[3].y), master_low);
+                    store4(o + 2 * ld, make_float4(a[0].z, a[1].z, a[2].z, a[3].z), master_low);
+                    store4(o + 3 * ld, make_float4(a[0].w, a[1].w, a[2].w, a[3].w), master_low);
+                }
+            }
+        }
+    } else {
+    // ---------------- products that write the caller's float64 P or its trace partials
     // row pass: each drain warp takes kBM / DW tile rows, lanes on column pairs; applies
     // beta C + D + shift and stores the entries with col >= row (all of them when not sym).
     // The C and D operands of G consecutive (row, column piece) iterations are loaded before
@@ -745,7 +873,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
             const bool w0 = !sym || gcol >= grow, w1 = !sym || gcol + 1 >= grow;
             double ta = 0.0;   // the diagonal entry, if this lane holds it
             float fa = 0.0f;
-            if constexpr (F64) {
+            {
                 const bool e0 = w0 && grow < n_real && gcol < n_real, e1 = w1 && grow < n_real && gcol + 1 < n_real;
                 double x0 = widen_f32(v0), x1 = widen_f32(v1);
                 float y0 = v0, y1 = v1;
@@ -765,7 +893,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
                 if (st.part) contrib(grow, gcol, x0, x1, y0, y1, e0, e1, ta, fa);
             }
             store_slot(grow, gcol, v0, v1, w0, w1, true);
-            if (F64 && st.part) {
+            if (st.part) {
                 // this (row, piece)'s sums (the `continue` above is uniform across the warp:
                 // tile widths are multiples of 128); pieces 2b, 2b + 1 form the tile's
                 // 128-column block b, added in that order by the warp that owns the row
@@ -789,7 +917,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
             }
         }
     }
-    if (F64 && st.part) {
+    if (st.part) {
         // the tile's 128 x 128 blocks: rows added in order; block (I, J) of the instance's
         // upper-block enumeration (row blocks in order, J >= I within a row)
         asm volatile("bar.sync 1, %0;" ::"n"(32 * DW) : "memory");
@@ -803,7 +931,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
             st.part[2 * blk + qty] = sacc;
         }
     }
-    if (!sym) return;
+    if (sym) {
     // Below the diagonal the solver's slots need only the 16-bit planes (operands of later
     // products, read by TMA as whole rows); every float32 master read (epilogue C and D,
     // moments, contraction) stays on or above the diagonal.
@@ -820,13 +948,13 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
         // outside the tile's diagonal block nothing below the diagonal is written, except
         // into the caller's float64 P, which is returned whole
         const bool slot_rows = !(ub && !lower_master && grow >= (int64_t)m0 + kBM);
-        if (!slot_rows && !(F64 && out64)) break;
+        if (!slot_rows && !out64) break;
 #pragma unroll
         for (int h = 0; h < kBM / 64; ++h) {
             const int r = h * 64 + 2 * lane;
             const int64_t gcol = (int64_t)m0 + r;   // output column
             const float v0 = tile[r * LD + c], v1 = tile[(r + 1) * LD + c];
-            if (F64 && out64) {
+            if (out64) {
                 // entries below the diagonal (counted twice by their mirrors above)
                 const bool e0 = grow > gcol && grow < n_real && gcol < n_real;
                 const bool e1 = grow > gcol + 1 && grow < n_real && gcol + 1 < n_real;
@@ -842,9 +970,8 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
             if (slot_rows) store_slot(grow, gcol, v0, v1, grow > gcol, grow > gcol + 1, lower_master);
         }
     }
-    };
-    if (out64 || st.part) passes(std::true_type{});
-    else passes(std::false_type{});
+    }
+    }
     if constexpr (CHAIN) {
         // this tile's stores are complete: release them to the next step's tiles (generic
         // stores read later through TMA: a proxy fence as well), then count the tile
