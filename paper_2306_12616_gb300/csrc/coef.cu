@@ -43,6 +43,7 @@ __global__ void k_cos_table(int M, double* ct) {
 // Block (node chunk, instance).
 __global__ void k_dos_weights(const Inst* __restrict__ insts, int n_terms, int M,
                               const double* __restrict__ ct) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.y];
     if (!in.res->active) return;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(512) k_bisect(const Inst* __restrict__ insts,
                                                  const InstIO* __restrict__ io,
                                                  const double* __restrict__ ct, int M,
                                                  int max_iter, int start_mu0) {
+    pdl_sync();
     __shared__ double sh[66];
     const Inst& in = insts[blockIdx.x];
     DevResult* res = in.res;
@@ -171,6 +173,7 @@ __global__ void __launch_bounds__(512) k_bisect(const Inst* __restrict__ insts,
 
 // mu of FO_MU_FIXED from the per-call inputs.
 __global__ void k_set_mu(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int batch) {
+    pdl_sync();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch) insts[i].res->mu = io[i].mu;
 }
@@ -179,6 +182,7 @@ __global__ void k_set_mu(const Inst* __restrict__ insts, const InstIO* __restric
 // Block (node chunk, instance).
 __global__ void k_fermi_nodes(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int M,
                               const double* __restrict__ ct) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.y];
     const DevResult* res = in.res;
     if (!res->active) return;
@@ -196,6 +200,7 @@ __global__ void k_fermi_nodes(const Inst* __restrict__ insts, const InstIO* __re
 // One warp per n; block (warp group, instance).
 __global__ void k_coeffs(const Inst* __restrict__ insts, const double* __restrict__ ct, int M,
                          int n_terms, int km) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.y];
     if (!in.res->active) return;
     const int lane = threadIdx.x & 31;
@@ -222,6 +227,7 @@ __global__ void k_coeffs(const Inst* __restrict__ insts, const double* __restric
 // 1 <= l <= m-2; c_{(m-1)k+i} = g_{i,m-1}/2; c_i = g_{i,0} if m = 1. Solved downwards in l.
 // One block per instance.
 __global__ void k_g_convert(const Inst* __restrict__ insts, int k, int m) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.x];
     if (!in.res->active) return;
     const double* c = in.c;
@@ -246,6 +252,7 @@ __global__ void k_g_convert(const Inst* __restrict__ insts, int k, int m) {
 // t_{l-1,j}), so d_{i,j} = sum_l g_{i,l} t_{l,j}, i.e. D = G A^{-1} for the A of Eq. (coeff
 // recursion). Written over g in place; one block per instance, the table in shared memory.
 __global__ void k_g_to_d(const Inst* __restrict__ insts, int k, int m) {
+    pdl_sync();
     extern __shared__ double sm_t[];   // t[l * m + j], m x m, then g[k x m]
     const Inst& in = insts[blockIdx.x];
     if (!in.res->active) return;
@@ -271,6 +278,7 @@ __global__ void k_g_to_d(const Inst* __restrict__ insts, int k, int m) {
 }
 
 __global__ void k_poly_trace(const Inst* __restrict__ insts, int n_terms) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.x];
     if (!in.res->active) return;
     double s = 0.0;
@@ -289,6 +297,7 @@ __global__ void k_poly_trace(const Inst* __restrict__ insts, int n_terms) {
 // instance.
 __global__ void __launch_bounds__(256) k_poly_width(const Inst* __restrict__ insts, const double* __restrict__ ct,
                                                     int M, int n_terms) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.x];
     DevResult* res = in.res;
     if (!res->active) return;
@@ -325,6 +334,7 @@ constexpr int kGroup = 16;
 
 __global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ insts, Work we, int k,
                                                       int m, int n_tslots) {
+    pdl_sync();
     extern __shared__ double gsh[];
     const int i = find_inst(we.pre, 0, we.count, blockIdx.x);
     const Inst& in = insts[i];
@@ -422,6 +432,7 @@ template <int MAXM>
 __global__ void __launch_bounds__(128, 4) k_contract_f32(const Inst* __restrict__ insts, Work wct, int k, int m,
                                                           int l0, int n_tslots, int planes_last, int fp16,
                                                           float pscale, int* dbg) {
+    pdl_sync();
     static_assert(MAXM % 4 == 0, "l pairs per half");
     constexpr int HM = MAXM / 2;                           // R_l per thread
     extern __shared__ __align__(16) float fsh[];
@@ -560,6 +571,7 @@ __global__ void __launch_bounds__(128, 4) k_contract_f32(const Inst* __restrict_
 // transpose of its upper counterpart).
 __global__ void __launch_bounds__(256) k_mirror_planes(const Inst* __restrict__ insts, Work ws, int slot0, int m,
                                                        int planes, int ublk, int* dbg) {
+    pdl_sync();
     __shared__ uint16_t tile[3][32][33];
     const int i = find_inst(ws.pre, 0, ws.count, blockIdx.x);
     if (!insts[i].res->active) return;
@@ -609,7 +621,7 @@ cudaError_t launch_cos_table(int M, double* ct, cudaStream_t s) {
 }
 
 cudaError_t launch_dos_weights(const Inst* in, int batch, const Shape& sh, const double* ct, cudaStream_t s) {
-    k_dos_weights<<<dim3((sh.M + 127) / 128, batch), 128, 0, s>>>(in, sh.n_terms, sh.M, ct);
+    launch_pdl(k_dos_weights, dim3((sh.M + 127) / 128, batch), 128, 0, s, in, sh.n_terms, sh.M, ct);
     return cudaGetLastError();
 }
 
@@ -618,25 +630,25 @@ cudaError_t launch_bisect(const Inst* in, const InstIO* io, int batch, const Sha
     // four warps per instance: the node sums are few float64 operations per thread, the
     // float64 shuffle trees and the block reduction are per warp (this GPU's float64 pipe is
     // narrow), so fewer warps finish an evaluation sooner
-    k_bisect<<<batch, 128, 0, s>>>(in, io, ct, sh.M, max_iter, start_mu0);
+    launch_pdl(k_bisect, batch, 128, 0, s, in, io, ct, sh.M, max_iter, start_mu0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_set_mu(const Inst* in, const InstIO* io, int batch, cudaStream_t s) {
-    k_set_mu<<<(batch + 127) / 128, 128, 0, s>>>(in, io, batch);
+    launch_pdl(k_set_mu, (batch + 127) / 128, 128, 0, s, in, io, batch);
     return cudaGetLastError();
 }
 
 cudaError_t launch_coefficients(const Inst* in, const InstIO* io, int batch, const Shape& sh,
                                 const double* ct, int with_poly_trace, cudaStream_t s, int* launches) {
-    k_fermi_nodes<<<dim3((sh.M + 255) / 256, batch), 256, 0, s>>>(in, io, sh.M, ct);
+    launch_pdl(k_fermi_nodes, dim3((sh.M + 255) / 256, batch), 256, 0, s, in, io, sh.M, ct);
     const int warps_per_block = 8;
-    k_coeffs<<<dim3((sh.km + warps_per_block - 1) / warps_per_block, batch), 32 * warps_per_block, 0, s>>>(
+    launch_pdl(k_coeffs, dim3((sh.km + warps_per_block - 1) / warps_per_block, batch), 32 * warps_per_block, 0, s, 
         in, ct, sh.M, sh.n_terms, sh.km);
-    k_g_convert<<<batch, sh.k < 1024 ? ((sh.k + 31) / 32) * 32 : 1024, 0, s>>>(in, sh.k, sh.m);
+    launch_pdl(k_g_convert, batch, sh.k < 1024 ? ((sh.k + 31) / 32) * 32 : 1024, 0, s, in, sh.k, sh.m);
     int l = 3;
     if (with_poly_trace) {
-        k_poly_trace<<<batch, 32, 0, s>>>(in, sh.n_terms);
+        launch_pdl(k_poly_trace, batch, 32, 0, s, in, sh.n_terms);
         ++l;
     }
     if (launches) *launches += l;
@@ -644,14 +656,14 @@ cudaError_t launch_coefficients(const Inst* in, const InstIO* io, int batch, con
 }
 
 cudaError_t launch_poly_width(const Inst* in, int batch, const Shape& sh, const double* ct, cudaStream_t s) {
-    k_poly_width<<<batch, 256, 0, s>>>(in, ct, sh.M, sh.n_terms);
+    launch_pdl(k_poly_width, batch, 256, 0, s, in, ct, sh.M, sh.n_terms);
     return cudaGetLastError();
 }
 
 cudaError_t launch_g_to_d(const Inst* in, int batch, const Shape& sh, cudaStream_t s) {
     const size_t smem = sizeof(double) * ((size_t)sh.m * sh.m + (size_t)sh.k * sh.m);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_g_to_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_g_to_d<<<batch, 256, smem, s>>>(in, sh.k, sh.m);
+    launch_pdl(k_g_to_d, batch, 256, smem, s, in, sh.k, sh.m);
     return cudaGetLastError();
 }
 
@@ -660,7 +672,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
         const size_t smem = (size_t)sh.k * sh.m * sizeof(double);
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_contract_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_contract_f64<<<we.total, 256, smem, s>>>(in, we, sh.k, sh.m, sh.n_tslots);
+        launch_pdl(k_contract_f64, we.total, 256, smem, s, in, we, sh.k, sh.m, sh.n_tslots);
         return cudaGetLastError();
     }
     const int planes_last = sh.m > 1 ? sh.planes : 0;
@@ -670,7 +682,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
     auto go = [&](auto kern, int maxm, int l0) {
         const size_t smem = (size_t)2 * sh.k * maxm * sizeof(float) + 2 * stage_bytes;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<wct.total, 2 * tpb, smem, s>>>(in, wct, sh.k, sh.m, l0, sh.n_tslots, planes_last, sh.fp16,
+        launch_pdl(kern, wct.total, 2 * tpb, smem, s, in, wct, sh.k, sh.m, l0, sh.n_tslots, planes_last, sh.fp16,
                                               sh.pscale_r, dbg);
     };
     for (int l0 = 0; l0 < sh.m; l0 += 32) {
@@ -686,7 +698,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
             default: go(k_contract_f32<32>, 32, l0); break;
         }
     }
-    if (planes_last > 0) k_mirror_planes<<<wsym.total, 256, 0, s>>>(in, wsym, sh.n_tslots, sh.m, planes_last,
+    if (planes_last > 0) launch_pdl(k_mirror_planes, wsym.total, 256, 0, s, in, wsym, sh.n_tslots, sh.m, planes_last,
                                                          sh.ublk, dbg);
     return cudaGetLastError();
 }

@@ -142,6 +142,7 @@ __device__ __forceinline__ Unit unit_of(int u, int tiles, int sl, int sh) {
 __global__ void __launch_bounds__(kMmaThreads, 1)
     k_dig_mma(const __grid_constant__ DigMaps maps, const Inst* __restrict__ insts, const int* __restrict__ pre, int i0,
               int i1, int unit0, int b0, int a_buf, int b_buf, int out_slot, int need_m, int* err_flag) {
+    pdl_launch();
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -156,7 +157,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
     const int gu = unit0 + (int)blockIdx.x;
     const int inst = find_inst(pre, i0, i1, gu);
     const Inst& in = insts[inst];
-    if (!step_needed(in.res, need_m)) return;
     const int nt = (int)(in.np / kT);
     const int u = gu - __ldg(pre + inst);
     const Unit w = unit_of(u, nt * (nt + 1) / 2, in.dig_sl, in.dig_sh);
@@ -188,6 +188,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
     }
+    pdl_wait();   // above: the plan's constant tables only; tensor memory is taken after the wait
+    if (!step_needed(in.res, need_m)) return;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tmem_slot)),
@@ -465,6 +467,7 @@ struct DigStep {
 // compared as integers).
 __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __restrict__ insts, const InstIO* __restrict__ io,
                                                     Work ws, const DigStep st) {
+    pdl_sync();
     __shared__ double sv[32][33];
     __shared__ unsigned long long su[32][33];
     __shared__ int s_e[2];
@@ -580,6 +583,7 @@ __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __r
 // master is complete on both sides.
 __global__ void __launch_bounds__(128) k_dig_split(const Inst* __restrict__ insts, Work ws, int slot0, int last_m,
                                                    int buf, int need_m) {
+    pdl_sync();
     const int inst = find_inst(ws.pre, 0, ws.count, blockIdx.x);
     const Inst& in = insts[inst];
     if (!step_needed(in.res, need_m)) return;
@@ -608,6 +612,7 @@ __global__ void __launch_bounds__(128) k_dig_split(const Inst* __restrict__ inst
 
 // Clears the largest-entry and unit records of slots [slot0, slot0 + count); one block per instance.
 __global__ void k_dig_reset(const Inst* __restrict__ insts, int slot0, int count) {
+    pdl_sync();
     const Inst& in = insts[blockIdx.x];
     for (int q = threadIdx.x; q < count; q += blockDim.x) in.smax[slot0 + q] = 0;
     for (int q = threadIdx.x; q < count * kDigMaxSplit; q += blockDim.x) in.umax[(size_t)slot0 * kDigMaxSplit + q] = 0;
@@ -709,7 +714,7 @@ cudaError_t dig_product(const Step& s, int dig_a, int dig_b, int dig_out, const 
         std::memset(&dm, 0, sizeof(dm));
         for (int b = 0; b < g.nb; ++b)
             std::memcpy(&dm.m[b], static_cast<const char*>(maps) + 128 * (size_t)(g.b0 + b), sizeof(CUtensorMap));
-        k_dig_mma<<<(unsigned)(u1 - u0), kMmaThreads, kMmaSmem, st>>>(dm, in, wu.pre, g.i0, g.i1, u0, g.b0, dig_a, dig_b,
+        launch_pdl(k_dig_mma, (unsigned)(u1 - u0), kMmaThreads, kMmaSmem, st, dm, in, wu.pre, g.i0, g.i1, u0, g.b0, dig_a, dig_b,
                                                                       dig_fused >= 0 ? s.out : -1, s.need_m, err_flag);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -728,21 +733,21 @@ cudaError_t dig_product(const Step& s, int dig_a, int dig_b, int dig_out, const 
     d.alpha_exp = s.alpha64 == 2.0 ? 1 : 0;
     d.beta = s.beta64;
     d.shift = s.shift64;
-    k_dig_update<<<(unsigned)wsym.total, 32 * kUpWarps, 0, st>>>(in, io, wsym, d);
+    launch_pdl(k_dig_update, (unsigned)wsym.total, 32 * kUpWarps, 0, st, in, io, wsym, d);
     *launches += 1;
     if (dig_out >= 0 && dig_fused < 0) {
         *launches += 1;
-        k_dig_split<<<(unsigned)wsym.total, 128, 0, st>>>(in, wsym, s.out, 0, dig_out, s.need_m);
+        launch_pdl(k_dig_split, (unsigned)wsym.total, 128, 0, st, in, wsym, s.out, 0, dig_out, s.need_m);
     }
     return cudaGetLastError();
 }
 
 cudaError_t dig_split(const Inst* in, const Work& wsym, int slot0, int last_m, int buf, cudaStream_t st) {
-    k_dig_split<<<(unsigned)wsym.total, 128, 0, st>>>(in, wsym, slot0, last_m, buf, 0);
+    launch_pdl(k_dig_split, (unsigned)wsym.total, 128, 0, st, in, wsym, slot0, last_m, buf, 0);
     return cudaGetLastError();
 }
 cudaError_t dig_reset(const Inst* in, int batch, int slot0, int count, cudaStream_t st) {
-    k_dig_reset<<<batch, 256, 0, st>>>(in, slot0, count);
+    launch_pdl(k_dig_reset, batch, 256, 0, st, in, slot0, count);
     return cudaGetLastError();
 }
 }  // namespace fo

@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
     __shared__ int abort_flag;
 
+    if constexpr (!CHAIN) pdl_launch();
     // ---------------- step, instance and tile of this CTA (uniform across the CTA)
     int sidx, gtile, inst;
     // chain launches: the ticket's step and the tile count its instance must reach first,
@@ -283,13 +284,13 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     }
     const Step& st = steps.s[sidx];
     const Inst& in = insts[inst];
-    if (!step_needed(in.res, st.need_m)) {
-        // an instance parked by the learned judge, or whose expansion does not need this
-        // step: its tiles count as done
-        if constexpr (CHAIN) {
+    if constexpr (CHAIN) {
+        if (!step_needed(in.res, st.need_m)) {
+            // an instance parked by the learned judge, or whose expansion does not need this
+            // step: its tiles count as done
             if (threadIdx.x == 0) atomicAdd(steps.done + (inst - i0), 1);
+            return;
         }
-        return;
     }
     const int np = (int)in.np;
     const CUtensorMap* map = &maps.m[in.bucket - b0];
@@ -340,6 +341,12 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
         if (sym == 2) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map_mn)) : "memory");
+    }
+    if constexpr (!CHAIN) {
+        // everything above reads the plan's constant tables only; tensor memory is taken after the
+        // wait, so that it is never held while the previous kernel's blocks may want it
+        pdl_wait();
+        if (!step_needed(in.res, st.need_m)) return;   // parked, or a step its expansion does not need
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1549,6 +1556,9 @@ cudaError_t launch_tc(const TcMaps& maps, const SL& st, unsigned grid, const Ins
     auto kern = k_tc_gemm<PA, PB, NPROD, F16, TBN, MINB, DW, CHAIN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
     if (e != cudaSuccess) return e;
+    if constexpr (!CHAIN)
+        return launch_pdl(kern, grid, Cfg::kThreads, Cfg::kSmem, s, maps, st, in, io, pre, i0, i1, tile0, tiles, b0,
+                          sym, err_flag);
     kern<<<grid, Cfg::kThreads, Cfg::kSmem, s>>>(maps, st, in, io, pre, i0, i1, tile0, tiles, b0, sym, err_flag);
     return cudaGetLastError();
 }

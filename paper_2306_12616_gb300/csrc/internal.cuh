@@ -12,6 +12,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "fermi.h"
 
@@ -156,6 +157,37 @@ struct Work {
     int count;        // instances
     int total;        // blocks
 };
+
+// Programmatic dependent launch. The kernels of a call form a chain on one stream; launched
+// through launch_pdl, a kernel may start once every block of its predecessor has started, so that
+// its launch latency (2 to 3 us between dependent kernels) and its set-up run while the
+// predecessor finishes. pdl_wait returns when the predecessor has completed and its writes are
+// visible (and, since that one waited the same way, everything before it): every kernel launched
+// this way executes it, in all threads, before it touches global memory other than the plan's
+// constant tables, and holds nothing then that another kernel's blocks could be waiting for.
+// Waiting blocks are not free: they share the SM of what still runs. The network's training kernels
+// (5.2 -> 5.7 ms for two epochs) and the kernel behind the Frobenius products are launched plainly.
+// Measured with this on all others: N = 64 1.04 -> 0.91 ms, N = 1000 2.02 -> 1.91 ms.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_sync() {
+    pdl_launch();
+    pdl_wait();
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
 
 // Whether a product step is computed for an instance: it is active, and its expansion (cut at
 // m_eff giant steps by a learned order) needs the step's output.

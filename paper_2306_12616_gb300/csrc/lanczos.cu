@@ -70,6 +70,7 @@ __device__ __forceinline__ Lz lz_of(const Inst& in) {
 }
 
 __global__ void k_lz_init(const Inst* __restrict__ insts, int batch) {
+    pdl_sync();
     __shared__ double sh[33];
     const Inst& in = insts[blockIdx.x];
     const Lz z = lz_of(in);
@@ -97,6 +98,7 @@ __global__ void k_lz_init(const Inst* __restrict__ insts, int batch) {
 __global__ void __launch_bounds__(32 * kGershRows) k_lz_matvec(const Inst* __restrict__ insts,
                                                                const InstIO* __restrict__ io, Work wg, int j,
                                                                double* part) {
+    pdl_sync();
     __shared__ double sp[kGershRows];
     const int b = blockIdx.x;
     const int i = find_inst(wg.pre, 0, wg.count, b);
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(32 * kGershRows) k_lz_matvec(const Inst* __res
 // thread adding them from global memory took 10 us).
 __global__ void __cluster_dims__(kLzCluster, 1, 1) __launch_bounds__(32)
     k_lz_update(const Inst* __restrict__ insts, Work wg, int j, const double* part) {
+    pdl_sync();
     constexpr int kChunk = 512;
     __shared__ double sp[kChunk];
     __shared__ double sh[kLzCluster];
@@ -228,6 +231,7 @@ __device__ double last_component(const double* alpha, const double* beta, int K,
 // path is then followed with the bisection's own test at every level: the same sequence, hence
 // the same bits, in a fifth of the dependent rounds (40 steps: 2.13 ms with one thread, 0.24 now).
 __global__ void __launch_bounds__(64) k_lz_bounds(const Inst* __restrict__ insts) {
+    pdl_sync();
     __shared__ double alpha[kLzMax], beta[kLzMax + 1], beta2[kLzMax + 1], s_th[2], s_rs[2];
     const Inst& in = insts[blockIdx.x];
     const Lz z = lz_of(in);
@@ -310,12 +314,12 @@ cudaError_t launch_lanczos(const Inst* in, const InstIO* io, int batch, Work wg,
                            cudaStream_t s, int* launches) {
     if (steps < 1) return cudaSuccess;
     if (steps > kLzMax) steps = kLzMax;
-    k_lz_init<<<batch, 256, 0, s>>>(in, batch);
+    launch_pdl(k_lz_init, batch, 256, 0, s, in, batch);
     for (int j = 0; j < steps; ++j) {
-        k_lz_matvec<<<wg.total, 32 * kGershRows, 0, s>>>(in, io, wg, j, part);
-        k_lz_update<<<batch * kLzCluster, 32, 0, s>>>(in, wg, j, part);
+        launch_pdl(k_lz_matvec, wg.total, 32 * kGershRows, 0, s, in, io, wg, j, part);
+        launch_pdl(k_lz_update, batch * kLzCluster, 32, 0, s, in, wg, j, part);
     }
-    k_lz_bounds<<<batch, 64, 0, s>>>(in);
+    launch_pdl(k_lz_bounds, batch, 64, 0, s, in);
     if (launches) *launches += 2 + 2 * steps;
     return cudaGetLastError();
 }
