@@ -10,7 +10,11 @@
 #include <type_traits>
 #include <cuda_fp16.h>
 
+#include <cooperative_groups.h>
+
 #include "internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace fo {
 namespace {
@@ -40,56 +44,121 @@ __global__ void k_cos_table(int M, double* ct) {
 
 // w_j = (1/M) (tau_0 + 2 sum_{n=1}^{n_terms-1} tau_n cos(n theta_j)), so that
 // sum_n c_n(mu) tau_n = sum_j f(e_j; mu) w_j for the interpolation coefficients c_n.
-// Block (node chunk, instance).
-__global__ void k_dos_weights(const Inst* __restrict__ insts, int n_terms, int M,
-                              const double* __restrict__ ct) {
+// Block (node chunk, instance). The float64 FMAs bound it (two lanes per clock and SM: 400 terms
+// take a warp 6400 clocks), and the cosines, one 8-byte gather per term and node: a single
+// instance therefore runs one warp per block (2048 nodes on 64 SMs), batches eight (the table is
+// then read by fewer blocks), and each block first copies the table to shared memory where it fits
+// (64 KB at M = 2048; kDosTable). 400 terms, one instance: 30 us with four warps per block reading
+// the table through L1, 51 with one.
+constexpr int kDosTable = 16384;   // largest table copied (entries): 128 KB
+constexpr int kDosLoads = 8;       // terms whose loads are issued together
+__global__ void __launch_bounds__(256) k_dos_weights(const Inst* __restrict__ insts, int n_terms, int M,
+                                                     const double* __restrict__ ct) {
+    extern __shared__ __align__(16) double dos_sm[];   // cosines (if copied), then the moments
+    const bool copied = 4 * (int64_t)M <= kDosTable;
+    const int64_t fourM = 4LL * M;
+    // the table is a constant of the plan: it may be read before the previous kernel has finished
+    if (copied) {
+        for (int q = threadIdx.x; q < (int)(fourM / 2); q += blockDim.x) cp_async16(dos_sm + 2 * q, ct + 2 * q);
+        cp_async_commit();
+    }
     pdl_sync();
     const Inst& in = insts[blockIdx.y];
-    if (!in.res->active) return;
+    const bool active = in.res->active != 0;
+    const int nt = active ? eff_terms(in.res, n_terms) : 0;
+    double* tau = dos_sm + (copied ? fourM : 0);
+    for (int n = threadIdx.x; n < nt; n += blockDim.x) tau[n] = in.tau[n];
+    cp_async_wait<0>();
+    __syncthreads();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= M) return;
-    const double* tau = in.tau;
-    const int64_t q = 2LL * j + 1, fourM = 4LL * M;
-    int64_t r = 0;
-    double s = 0.0;
-    const int nt = eff_terms(in.res, n_terms);
-    for (int n = 1; n < nt; ++n) {
-        r += q;
-        if (r >= fourM) r -= fourM;
-        s = fma(tau[n], ct[r], s);
-    }
+    if (!active || j >= M) return;
+    auto sum = [&](const double* c, auto index) {
+        using I = decltype(index);   // 32 bits for a copied table
+        const I q = 2 * (I)j + 1, period = (I)fourM;
+        I x = 0;
+        double s = 0.0;
+        int n = 1;
+        for (; n + kDosLoads <= nt; n += kDosLoads) {
+            double v[kDosLoads];
+#pragma unroll
+            for (int u = 0; u < kDosLoads; ++u) {
+                x += q;
+                if (x >= period) x -= period;
+                v[u] = c[x];
+            }
+#pragma unroll
+            for (int u = 0; u < kDosLoads; ++u) s = fma(tau[n + u], v[u], s);
+        }
+        for (; n < nt; ++n) {
+            x += q;
+            if (x >= period) x -= period;
+            s = fma(tau[n], c[x], s);
+        }
+        return s;
+    };
+    const double s = copied ? sum(dos_sm, int{}) : sum(ct, int64_t{});
     in.w[j] = (tau[0] + 2.0 * s) / (double)M;
 }
 
-// F(mu) + N_e = sum_j w_j f(e_j; mu) and dF/dmu = sum_j w_j f_j (1 - f_j) / kT over the M
-// nodes, fixed summation order, both broadcast to the block.
-__device__ void trace_at(double mu, const double* __restrict__ w, const double* __restrict__ ct,
-                         int M, double mid, double half, double inv2kT, double* sh, double* tr,
-                         double* dtr) {
+// F(mu) + N_e = sum_j w_j f(e_j; mu) and dF/dmu = sum_j w_j f_j (1 - f_j) / kT over the M nodes.
+// Thread t of the cluster's 32 kMuCluster takes nodes t, t + 32 kMuCluster, ...; warp trees, then the
+// warps' sums in order, exchanged through distributed shared memory (buffer `par`, alternating
+// between calls so that one cluster barrier per evaluation is enough). Every thread gets the result.
+constexpr int kMuCluster = 4;       // one-warp blocks per instance
+constexpr int kMuNodes = 32;        // nodes per thread held in shared memory (up to M = 4096)
+struct MuNodes {
+    double e[kMuNodes][32], w[kMuNodes][32];
+};
+__device__ __forceinline__ void trace_at(double mu, const MuNodes& nd, const double* __restrict__ w,
+                                         const double* __restrict__ ct, int M, double mid, double half, double inv2kT,
+                                         double (*sh)[2 * kMuCluster], int& par, int rank, double* tr, double* dtr) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x, t = rank * 32 + lane;
     double s = 0.0, d = 0.0;
-    for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        const double f = fermi(mid + half * ct[2 * j + 1], mu, inv2kT);
-        s = fma(w[j], f, s);
-        d = fma(w[j], f * (1.0 - f), d);
+    // (a node of f = 0 or 1 exactly adds nothing to the derivative)
+    auto add = [&](double e, double wj) {
+        const double x = (e - mu) * inv2kT;
+        const long long xb = __double_as_longlong(x);
+        if (xb >= 0x4034000000000000ll && xb < 0x7ff0000000000001ll) {   // x >= 20: f = 0
+            s = fma(wj, 0.0, s);
+            return;
+        }
+        if ((unsigned long long)xb >= 0xc034000000000000ull && (unsigned long long)xb < 0xfff0000000000001ull) {
+            s = s + wj;   // x <= -20: f = 1
+            return;
+        }
+        const double f = 0.5 - 0.5 * tanh(x);
+        s = fma(wj, f, s);
+        d = fma(wj, f * (1.0 - f), d);
+    };
+#pragma unroll 1
+    for (int i = 0; i < kMuNodes; ++i) {
+        if (t + i * 32 * kMuCluster >= M) break;
+        add(nd.e[i][lane], nd.w[i][lane]);
     }
+    for (int j = t + kMuNodes * 32 * kMuCluster; j < M; j += 32 * kMuCluster) add(mid + half * ct[2 * j + 1], w[j]);
     s = warp_sum(s);
     d = warp_sum(d);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (lane == 0) { sh[warp] = s; sh[32 + warp] = d; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0, u = 0.0;
-        for (int i = 0; i < nw; ++i) { t += sh[i]; u += sh[32 + i]; }
-        sh[64] = t;
-        sh[65] = u * 2.0 * inv2kT;
+    if (lane < kMuCluster) {
+        double* dst = cl.map_shared_rank(&sh[par][0], lane);
+        dst[2 * rank] = s;
+        dst[2 * rank + 1] = d;
     }
-    __syncthreads();
-    *tr = sh[64];
-    if (dtr) *dtr = sh[65];
+    cl.sync();
+    double ts = 0.0, td = 0.0;
+#pragma unroll
+    for (int i = 0; i < kMuCluster; ++i) {
+        ts += sh[par][2 * i];
+        td += sh[par][2 * i + 1];
+    }
+    par ^= 1;
+    *tr = ts;
+    if (dtr) *dtr = td * 2.0 * inv2kT;
 }
 
-// Root of F(mu) = sum_n c_n(mu) tau_n - N_e, one block per instance. Bracket [emin, emax],
+// Root of F(mu) = sum_n c_n(mu) tau_n - N_e, one cluster of four one-warp blocks per instance (the
+// float64 operations of an evaluation on four SMs instead of one, the nodes' energies and weights in
+// shared memory). Bracket [emin, emax],
 // widened by 10 kT (at most 8 times per side). Inside the bracket a Newton step on the
 // exact derivative of the node sum is taken when it stays in the bracket and is at most
 // half the step before the last one, a halving otherwise; the bracket shrinks with the sign
@@ -98,36 +167,48 @@ __device__ void trace_at(double mu, const double* __restrict__ w, const double* 
 // bracket (the learned proposal). Stop when |F| <= 1e-12 max(1, N_e) (mu = that point) or
 // the bracket is narrower than 1e-15 (emax - emin) (mu = midpoint), at most max_iter
 // evaluations.
-__global__ void __launch_bounds__(512) k_bisect(const Inst* __restrict__ insts,
+__global__ void __cluster_dims__(kMuCluster, 1, 1) __launch_bounds__(32) k_bisect(const Inst* __restrict__ insts,
                                                  const InstIO* __restrict__ io,
                                                  const double* __restrict__ ct, int M,
                                                  int max_iter, int start_mu0) {
     pdl_sync();
-    __shared__ double sh[66];
-    const Inst& in = insts[blockIdx.x];
+    __shared__ double sh[2][2 * kMuCluster];
+    cg::cluster_group cl = cg::this_cluster();
+    const int i0 = (int)blockIdx.x / kMuCluster, rank = (int)cl.block_rank();
+    const Inst& in = insts[i0];
     DevResult* res = in.res;
-    if (!res->active) return;
+    if (!res->active) return;   // uniform over the cluster
+    cl.sync();                  // every block runs before its shared memory is written
+    int par = 0;
     const double* w = in.w;
-    const double kT = io[blockIdx.x].kT, n_e = io[blockIdx.x].n_e;
+    const double kT = io[i0].kT, n_e = io[i0].n_e;
     const double ea = res->bounds[0], eb = res->bounds[1];
     const double mid = 0.5 * (eb + ea), half = 0.5 * (eb - ea), inv2kT = 0.5 / kT;
+    __shared__ MuNodes nd;   // each thread reads only what it wrote
+#pragma unroll 8
+    for (int i = 0; i < kMuNodes; ++i) {
+        const int j = rank * 32 + (int)threadIdx.x + i * 32 * kMuCluster;
+        if (j >= M) break;
+        nd.e[i][threadIdx.x] = mid + half * ct[2 * j + 1];
+        nd.w[i][threadIdx.x] = w[j];
+    }
     double lo = ea, hi = eb, t;
     // F at the bracket ends, from the widening loops (evaluated again only where a loop ended
     // by widening past its last evaluation)
     double flo = 1.0, fhi = -1.0;
     bool have_lo = false, have_hi = false;
     for (int q = 0; q < 8; ++q) {
-        trace_at(lo, w, ct, M, mid, half, inv2kT, sh, &t, nullptr);
+        trace_at(lo, nd, w, ct, M, mid, half, inv2kT, sh, par, rank, &t, nullptr);
         if (t - n_e <= 0.0) { flo = t - n_e; have_lo = true; break; }
         lo -= 10.0 * kT;
     }
     for (int q = 0; q < 8; ++q) {
-        trace_at(hi, w, ct, M, mid, half, inv2kT, sh, &t, nullptr);
+        trace_at(hi, nd, w, ct, M, mid, half, inv2kT, sh, par, rank, &t, nullptr);
         if (t - n_e >= 0.0) { fhi = t - n_e; have_hi = true; break; }
         hi += 10.0 * kT;
     }
-    if (!have_lo) { trace_at(lo, w, ct, M, mid, half, inv2kT, sh, &flo, nullptr); flo -= n_e; }
-    if (!have_hi) { trace_at(hi, w, ct, M, mid, half, inv2kT, sh, &fhi, nullptr); fhi -= n_e; }
+    if (!have_lo) { trace_at(lo, nd, w, ct, M, mid, half, inv2kT, sh, par, rank, &flo, nullptr); flo -= n_e; }
+    if (!have_hi) { trace_at(hi, nd, w, ct, M, mid, half, inv2kT, sh, par, rank, &fhi, nullptr); fhi -= n_e; }
     int status = FO_OK, iters = 0;
     double mu = 0.5 * (lo + hi);
     if (flo > 0.0 || fhi < 0.0) {
@@ -145,7 +226,7 @@ __global__ void __launch_bounds__(512) k_bisect(const Inst* __restrict__ insts,
         double dx = hi - lo, dxold = dx;
         for (int it = 1; it <= max_iter; ++it) {
             double f, df;
-            trace_at(x, w, ct, M, mid, half, inv2kT, sh, &f, &df);
+            trace_at(x, nd, w, ct, M, mid, half, inv2kT, sh, par, rank, &f, &df);
             f -= n_e;
             iters = it;
             if (fabs(f) <= tol_f) { mu = x; done = true; break; }
@@ -162,7 +243,8 @@ __global__ void __launch_bounds__(512) k_bisect(const Inst* __restrict__ insts,
             status = FO_ERR_NOT_CONVERGED;
         }
     }
-    if (threadIdx.x == 0) {
+    cl.sync();   // no block leaves while another may write its shared memory or read the record
+    if (rank == 0 && threadIdx.x == 0) {
         res->mu = mu;
         res->iters = iters;
         res->mu_lo = lo;
@@ -197,7 +279,9 @@ __global__ void k_fermi_nodes(const Inst* __restrict__ insts, const InstIO* __re
 }
 
 // c_n = (2 - delta_{n0}) / M sum_j f_j cos(n theta_j) for n < n_terms, 0 for n_terms <= n < km.
-// One warp per n; block (warp group, instance).
+// One warp per n; block (warp group, instance): two warps per block, so that the float64 FMAs, which
+// bound it, spread over the SMs.
+constexpr int kCoefLoads = 8;
 __global__ void k_coeffs(const Inst* __restrict__ insts, const double* __restrict__ ct, int M,
                          int n_terms, int km) {
     pdl_sync();
@@ -212,11 +296,29 @@ __global__ void k_coeffs(const Inst* __restrict__ insts, const double* __restric
         return;
     }
     const double* f = in.f;
+    // r = n (2 j + 1) mod 4M, advanced by 64 n mod 4M from one of the lane's nodes to the next (a
+    // 64-bit division per node took most of the kernel's time)
     const int64_t fourM = 4LL * M;
+    const int64_t step = (64LL * n) % fourM;
+    int64_t r = ((int64_t)n * (2LL * lane + 1)) % fourM;
     double s = 0.0;
-    for (int j = lane; j < M; j += 32) {
-        const int64_t r = ((int64_t)n * (2LL * j + 1)) % fourM;
+    int j = lane;
+    for (; j + 32 * (kCoefLoads - 1) < M; j += 32 * kCoefLoads) {
+        double c[kCoefLoads], v[kCoefLoads];
+#pragma unroll
+        for (int u = 0; u < kCoefLoads; ++u) {
+            c[u] = __ldg(ct + r);
+            v[u] = f[j + 32 * u];
+            r += step;
+            if (r >= fourM) r -= fourM;
+        }
+#pragma unroll
+        for (int u = 0; u < kCoefLoads; ++u) s = fma(v[u], c[u], s);
+    }
+    for (; j < M; j += 32) {
         s = fma(f[j], ct[r], s);
+        r += step;
+        if (r >= fourM) r -= fourM;
     }
     s = warp_sum(s);
     if (lane == 0) c[n] = (n == 0 ? 1.0 : 2.0) * s / (double)M;
@@ -225,12 +327,19 @@ __global__ void k_coeffs(const Inst* __restrict__ insts, const double* __restric
 // Giant-step coefficients from c (zero-padded to km), g stored l-major: g[l*k + i].
 // c_{lk} = g_{0,l}; c_i = g_{i,0} + g_{k-i,1}/2; c_{lk+i} = (g_{i,l} + g_{k-i,l+1})/2 for
 // 1 <= l <= m-2; c_{(m-1)k+i} = g_{i,m-1}/2; c_i = g_{i,0} if m = 1. Solved downwards in l.
-// One block per instance.
-__global__ void k_g_convert(const Inst* __restrict__ insts, int k, int m) {
+// One block per instance, the coefficients and the g of one l at a time in shared memory (a step of
+// dependent global loads per l took 10 us at m = 20). With poly_trace, warp 0 then also forms
+// sum_n c_n tau_n.
+__global__ void k_g_convert(const Inst* __restrict__ insts, int k, int m, int n_terms, int poly_trace) {
     pdl_sync();
+    extern __shared__ double cs[];   // c (k m), then two rows of g
     const Inst& in = insts[blockIdx.x];
     if (!in.res->active) return;
-    const double* c = in.c;
+    const double* c = cs;
+    double* gn = cs + k * m;         // g of l + 1
+    double* gl = gn + k;             // g of l
+    for (int q = threadIdx.x; q < k * m; q += blockDim.x) cs[q] = in.c[q];
+    __syncthreads();
     double* g = in.g;
     for (int l = m - 1; l >= 0; --l) {
         for (int i = threadIdx.x; i < k; i += blockDim.x) {
@@ -238,11 +347,23 @@ __global__ void k_g_convert(const Inst* __restrict__ insts, int k, int m) {
             double v;
             if (i == 0 || m == 1) v = ci;
             else if (l == m - 1) v = 2.0 * ci;
-            else if (l == 0) v = ci - 0.5 * g[1 * k + (k - i)];
-            else v = 2.0 * ci - g[(l + 1) * k + (k - i)];
+            else if (l == 0) v = ci - 0.5 * gn[k - i];
+            else v = 2.0 * ci - gn[k - i];
+            gl[i] = v;
             g[l * k + i] = v;
         }
         __syncthreads();
+        double* t = gn;
+        gn = gl;
+        gl = t;
+    }
+    if (poly_trace && threadIdx.x < 32) {
+        double s = 0.0;
+        const int nt = eff_terms(in.res, n_terms);
+#pragma unroll 4
+        for (int n = threadIdx.x; n < nt; n += 32) s = fma(c[n], in.tau[n], s);
+        s = warp_sum(s);
+        if (threadIdx.x == 0) in.res->trace_poly = s;
     }
 }
 
@@ -275,17 +396,6 @@ __global__ void k_g_to_d(const Inst* __restrict__ insts, int k, int m) {
         for (int l = j; l < m; ++l) s = fma(gs[l * k + i], t[l * m + j], s);
         in.g[j * k + i] = s;
     }
-}
-
-__global__ void k_poly_trace(const Inst* __restrict__ insts, int n_terms) {
-    pdl_sync();
-    const Inst& in = insts[blockIdx.x];
-    if (!in.res->active) return;
-    double s = 0.0;
-    const int nt = eff_terms(in.res, n_terms);
-    for (int n = threadIdx.x; n < nt; n += 32) s = fma(in.c[n], in.tau[n], s);
-    s = warp_sum(s);
-    if (threadIdx.x == 0) in.res->trace_poly = s;
 }
 
 // Effective temperature of the truncated expansion p(e) = sum_n c_n T_n(x(e)) at the current
@@ -621,49 +731,52 @@ cudaError_t launch_cos_table(int M, double* ct, cudaStream_t s) {
 }
 
 cudaError_t launch_dos_weights(const Inst* in, int batch, const Shape& sh, const double* ct, cudaStream_t s) {
-    launch_pdl(k_dos_weights, dim3((sh.M + 127) / 128, batch), 128, 0, s, in, sh.n_terms, sh.M, ct);
+    const int threads = batch <= kSmallBatch ? 32 : 256;
+    const size_t table = 4 * (int64_t)sh.M <= kDosTable ? 4 * (size_t)sh.M : 0;
+    const size_t smem = sizeof(double) * (table + sh.n_terms);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_dos_weights, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(double) * (kDosTable + 4096)));
+        if (e != cudaSuccess) return e;
+    }
+    launch_pdl(batch, k_dos_weights, dim3((sh.M + threads - 1) / threads, batch), threads, smem, s, in, sh.n_terms, sh.M, ct);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bisect(const Inst* in, const InstIO* io, int batch, const Shape& sh, const double* ct,
                           int max_iter, int start_mu0, cudaStream_t s) {
-    // four warps per instance: the node sums are few float64 operations per thread, the
-    // float64 shuffle trees and the block reduction are per warp (this GPU's float64 pipe is
-    // narrow), so fewer warps finish an evaluation sooner
-    launch_pdl(k_bisect, batch, 128, 0, s, in, io, ct, sh.M, max_iter, start_mu0);
+    launch_pdl(batch, k_bisect, batch * kMuCluster, 32, 0, s, in, io, ct, sh.M, max_iter, start_mu0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_set_mu(const Inst* in, const InstIO* io, int batch, cudaStream_t s) {
-    launch_pdl(k_set_mu, (batch + 127) / 128, 128, 0, s, in, io, batch);
+    launch_pdl(batch, k_set_mu, (batch + 127) / 128, 128, 0, s, in, io, batch);
     return cudaGetLastError();
 }
 
 cudaError_t launch_coefficients(const Inst* in, const InstIO* io, int batch, const Shape& sh,
                                 const double* ct, int with_poly_trace, cudaStream_t s, int* launches) {
-    launch_pdl(k_fermi_nodes, dim3((sh.M + 255) / 256, batch), 256, 0, s, in, io, sh.M, ct);
-    const int warps_per_block = 8;
-    launch_pdl(k_coeffs, dim3((sh.km + warps_per_block - 1) / warps_per_block, batch), 32 * warps_per_block, 0, s, 
+    launch_pdl(batch, k_fermi_nodes, dim3((sh.M + 255) / 256, batch), 256, 0, s, in, io, sh.M, ct);
+    const int warps_per_block = 2;
+    launch_pdl(batch, k_coeffs, dim3((sh.km + warps_per_block - 1) / warps_per_block, batch), 32 * warps_per_block, 0, s, 
         in, ct, sh.M, sh.n_terms, sh.km);
-    launch_pdl(k_g_convert, batch, sh.k < 1024 ? ((sh.k + 31) / 32) * 32 : 1024, 0, s, in, sh.k, sh.m);
-    int l = 3;
-    if (with_poly_trace) {
-        launch_pdl(k_poly_trace, batch, 32, 0, s, in, sh.n_terms);
-        ++l;
-    }
+    const size_t smem = sizeof(double) * ((size_t)sh.km + 2 * sh.k);
+    launch_pdl(batch, k_g_convert, batch, sh.k < 32 ? 32 : ((sh.k + 31) / 32) * 32, smem, s, in, sh.k, sh.m, sh.n_terms,
+               with_poly_trace);
+    const int l = 3;
     if (launches) *launches += l;
     return cudaGetLastError();
 }
 
 cudaError_t launch_poly_width(const Inst* in, int batch, const Shape& sh, const double* ct, cudaStream_t s) {
-    launch_pdl(k_poly_width, batch, 256, 0, s, in, ct, sh.M, sh.n_terms);
+    launch_pdl(batch, k_poly_width, batch, 256, 0, s, in, ct, sh.M, sh.n_terms);
     return cudaGetLastError();
 }
 
 cudaError_t launch_g_to_d(const Inst* in, int batch, const Shape& sh, cudaStream_t s) {
     const size_t smem = sizeof(double) * ((size_t)sh.m * sh.m + (size_t)sh.k * sh.m);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_g_to_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(k_g_to_d, batch, 256, smem, s, in, sh.k, sh.m);
+    launch_pdl(batch, k_g_to_d, batch, 256, smem, s, in, sh.k, sh.m);
     return cudaGetLastError();
 }
 
@@ -672,7 +785,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
         const size_t smem = (size_t)sh.k * sh.m * sizeof(double);
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_contract_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(k_contract_f64, we.total, 256, smem, s, in, we, sh.k, sh.m, sh.n_tslots);
+        launch_pdl(we.count, k_contract_f64, we.total, 256, smem, s, in, we, sh.k, sh.m, sh.n_tslots);
         return cudaGetLastError();
     }
     const int planes_last = sh.m > 1 ? sh.planes : 0;
@@ -682,7 +795,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
     auto go = [&](auto kern, int maxm, int l0) {
         const size_t smem = (size_t)2 * sh.k * maxm * sizeof(float) + 2 * stage_bytes;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(kern, wct.total, 2 * tpb, smem, s, in, wct, sh.k, sh.m, l0, sh.n_tslots, planes_last, sh.fp16,
+        launch_pdl(wct.count, kern, wct.total, 2 * tpb, smem, s, in, wct, sh.k, sh.m, l0, sh.n_tslots, planes_last, sh.fp16,
                                               sh.pscale_r, dbg);
     };
     for (int l0 = 0; l0 < sh.m; l0 += 32) {
@@ -698,7 +811,7 @@ cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const 
             default: go(k_contract_f32<32>, 32, l0); break;
         }
     }
-    if (planes_last > 0) launch_pdl(k_mirror_planes, wsym.total, 256, 0, s, in, wsym, sh.n_tslots, sh.m, planes_last,
+    if (planes_last > 0) launch_pdl(wsym.count, k_mirror_planes, wsym.total, 256, 0, s, in, wsym, sh.n_tslots, sh.m, planes_last,
                                                          sh.ublk, dbg);
     return cudaGetLastError();
 }

@@ -725,7 +725,10 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     if (to_slot) {
         float4* t4 = reinterpret_cast<float4*>(smem);
         const bool master_low = st.lower_master != 0;
-        auto store4 = [&](int64_t o, float4 v, bool master) {
+        // 32-bit offsets from a 64-bit base: within the tile's rows, or the mirrored rows
+        const int ldi = np;
+        auto store4 = [&](int64_t base_o, int off, float4 v, bool master) {
+            const int64_t o = base_o + off;
             if (!FO_CHK(st.dbg, o >= 0 && o + 4 <= ld * ld && (o & 3) == 0, 112, o / ld, o % ld)) return;
             if (master) *reinterpret_cast<float4*>(out_x + o) = v;
             if (planes > 0) {
@@ -749,20 +752,23 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
         constexpr int RPW = kBM / DW, NB = TBN / kBM, NIT = RPW * NB;
         constexpr int G = (DW == 16 || MINB == 2) ? 4 : 8;
         static_assert(NIT % G == 0, "row-pass groups");
+        const int64_t tile_o = (int64_t)m0 * ld + n0 + 4 * lane;   // this lane's columns of the tile's first row
 #pragma unroll 1
         for (int q0 = 0; q0 < NIT; q0 += G) {
             float4 cv[G], dv[G];
+            const float* cp = Cm + tile_o;
+            const float* dp = Dm + tile_o;
 #pragma unroll
             for (int u = 0; u < G; ++u) {
                 const int q = q0 + u, r = ew * RPW + q / NB, b = q % NB;
-                const int64_t o = ((int64_t)m0 + r) * ld + n0 + b * kBM + 4 * lane;
+                const int o = r * ldi + b * kBM;
                 cv[u] = dv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (b < nbox) {
                     // within a chain launch other SMs wrote C and D during this launch: L2 loads
-                    if (Cm) cv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(Cm + o))
-                                          : *reinterpret_cast<const float4*>(Cm + o);
-                    if (Dm) dv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(Dm + o))
-                                          : *reinterpret_cast<const float4*>(Dm + o);
+                    if (Cm) cv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(cp + o))
+                                          : *reinterpret_cast<const float4*>(cp + o);
+                    if (Dm) dv[u] = CHAIN ? __ldcg(reinterpret_cast<const float4*>(dp + o))
+                                          : *reinterpret_cast<const float4*>(dp + o);
                 }
             }
 #pragma unroll
@@ -783,16 +789,18 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
                     v.z += dv[u].z;
                     v.w += dv[u].w;
                 }
-                const int64_t grow = (int64_t)m0 + r, gcol = (int64_t)n0 + b * kBM + 4 * lane;
-                if (grow < n_real) {
-                    if (gcol == grow) v.x += st.shift;
-                    if (gcol + 1 == grow) v.y += st.shift;
-                    if (gcol + 2 == grow) v.z += st.shift;
-                    if (gcol + 3 == grow) v.w += st.shift;
+                if (n0 + b * kBM == m0) {   // a block on the diagonal
+                    const int e = r - 4 * lane;
+                    if ((e & ~3) == 0 && m0 + r < n_real) {
+                        if (e == 0) v.x += st.shift;
+                        if (e == 1) v.y += st.shift;
+                        if (e == 2) v.z += st.shift;
+                        if (e == 3) v.w += st.shift;
+                    }
                 }
                 const bool dblk = has_diag && b == 0;
                 if (dblk || mirror) *tw = v;
-                if (!dblk) store4(grow * ld + gcol, v, true);
+                if (!dblk) store4(tile_o, r * ldi + b * kBM, v, true);
             }
         }
         if (sym) {
@@ -808,20 +816,21 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
                     if (c + 1 < r) v.y = low(1);
                     if (c + 2 < r) v.z = low(2);
                     if (c + 3 < r) v.w = low(3);
-                    store4(((int64_t)m0 + r) * ld + n0 + c, v, true);
+                    store4(tile_o, r * ldi, v, true);
                 }
             }
             if (mirror) {
                 // four output rows n0 + c .. + 3 at a time: lanes on four neighbouring tile rows each
+                const int64_t mir_o = (int64_t)n0 * ld + m0 + 4 * lane;
                 for (int g4 = ew + (has_diag ? kBM / 4 : 0); g4 < nbox * (kBM / 4); g4 += DW) {
                     float4 a[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) a[i] = t4[slot_word<TBN>(4 * lane + i, g4)];
-                    const int64_t o = ((int64_t)n0 + 4 * g4) * ld + m0 + 4 * lane;
-                    store4(o, make_float4(a[0].x, a[1].x, a[2].x, a[3].x), master_low);
-                    store4(o + ld, make_float4(a[0].y, a[1].y, a[2].y, a[3].y), master_low);
-                    store4(o + 2 * ld, make_float4(a[0].z, a[1].z, a[2].z, a[3].z), master_low);
-                    store4(o + 3 * ld, make_float4(a[0].w, a[1].w, a[2].w, a[3].w), master_low);
+                    const int o = 4 * g4 * ldi;
+                    store4(mir_o, o, make_float4(a[0].x, a[1].x, a[2].x, a[3].x), master_low);
+                    store4(mir_o, o + ldi, make_float4(a[0].y, a[1].y, a[2].y, a[3].y), master_low);
+                    store4(mir_o, o + 2 * ldi, make_float4(a[0].z, a[1].z, a[2].z, a[3].z), master_low);
+                    store4(mir_o, o + 3 * ldi, make_float4(a[0].w, a[1].w, a[2].w, a[3].w), master_low);
                 }
             }
         }

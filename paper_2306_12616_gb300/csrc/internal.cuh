@@ -174,6 +174,10 @@ __device__ __forceinline__ void pdl_sync() {
     pdl_launch();
     pdl_wait();
 }
+// Of small-batch launches (launch_pdl with a batch), the kernels between the products are dependent
+// programmatically only up to this many instances: beyond it they are long enough to hide a launch,
+// and what waits beside them costs more (512 instances: 34.9 -> 35.9 ms).
+constexpr int kSmallBatch = 4;
 template <class... P, class... A>
 cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t cfg = {};
@@ -187,6 +191,14 @@ cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, c
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+template <class... P, class... A>
+cudaError_t launch_pdl(int batch, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       A&&... args) {
+    if (batch <= kSmallBatch) return launch_pdl(kern, grid, block, smem, s, std::forward<A>(args)...);
+    kern<<<grid, block, smem, s>>>(std::forward<A>(args)...);
+    return cudaGetLastError();
 }
 
 // Whether a product step is computed for an instance: it is active, and its expansion (cut at

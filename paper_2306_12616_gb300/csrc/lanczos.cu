@@ -314,12 +314,12 @@ cudaError_t launch_lanczos(const Inst* in, const InstIO* io, int batch, Work wg,
                            cudaStream_t s, int* launches) {
     if (steps < 1) return cudaSuccess;
     if (steps > kLzMax) steps = kLzMax;
-    launch_pdl(k_lz_init, batch, 256, 0, s, in, batch);
+    launch_pdl(batch, k_lz_init, batch, 256, 0, s, in, batch);
     for (int j = 0; j < steps; ++j) {
-        launch_pdl(k_lz_matvec, wg.total, 32 * kGershRows, 0, s, in, io, wg, j, part);
-        launch_pdl(k_lz_update, batch * kLzCluster, 32, 0, s, in, wg, j, part);
+        launch_pdl(batch, k_lz_matvec, wg.total, 32 * kGershRows, 0, s, in, io, wg, j, part);
+        launch_pdl(batch, k_lz_update, batch * kLzCluster, 32, 0, s, in, wg, j, part);
     }
-    launch_pdl(k_lz_bounds, batch, 64, 0, s, in);
+    launch_pdl(batch, k_lz_bounds, batch, 64, 0, s, in);
     if (launches) *launches += 2 + 2 * steps;
     return cudaGetLastError();
 }

@@ -924,24 +924,33 @@ __global__ void k_sum_partials(const Inst* __restrict__ insts, int npairs, int o
 // (T_{lk}, l = 2..m-1) and gram[(l-1)*(k-1) + (i-1)] = <T_{lk}, T_i> (l = 1..m-1,
 // i = 1..k-1) through tau_{lk+i} = 2 <T_{lk}, T_i> - tau_{lk-i} (Eq. identity).
 // Within one l the k - 1 moments are independent (tau_{lk-i} belongs to the range of l - 1):
-// threads take i, the block steps through l (a serial loop of dependent global loads took
-// tens of microseconds).
-__global__ void k_assemble_moments(const Inst* __restrict__ insts, int k, int m, int n_terms) {
+// threads take i, the block steps through l, the moments of the last l in shared memory and the
+// Frobenius products of the next one already requested (steps of dependent global loads took 11 us
+// at m = 20). k <= 64 (one thread per i).
+__global__ void __launch_bounds__(64) k_assemble_moments(const Inst* __restrict__ insts, int k, int m, int n_terms) {
     pdl_sync();
+    __shared__ double row[2][65];   // tau_{(l-1)k .. lk} and tau_{lk .. (l+1)k}
     const Inst& in = insts[blockIdx.x];
     if (!in.res->active) return;
     const double* diag = in.diag;
     const double* gram = in.gram;
     double* tau = in.tau;
-    if (threadIdx.x == 0) tau[0] = (double)in.n;
-    for (int i = 1 + (int)threadIdx.x; i <= k && i < n_terms; i += blockDim.x) tau[i] = diag[i - 1];
+    const int i = threadIdx.x;
+    auto product = [&](int l) { return i >= 1 && i < k && l < m ? gram[(l - 1) * (k - 1) + (i - 1)] : 0.0; };
+    double next = product(1);
+    if (i == 0) tau[0] = row[0][0] = (double)in.n;
+    for (int q = 1 + i; q <= k && q < n_terms; q += blockDim.x) tau[q] = row[0][q] = diag[q - 1];
+    if (i == 0 && k < n_terms) row[1][0] = diag[k - 1];
     __syncthreads();
     for (int l = 1; l < m; ++l) {
         const int base = l * k;
         if (base >= n_terms) break;
-        if (l >= 2 && threadIdx.x == 0) tau[base] = diag[k + l - 2];
-        for (int i = 1 + (int)threadIdx.x; i < k && base + i < n_terms; i += blockDim.x)
-            tau[base + i] = 2.0 * gram[(l - 1) * (k - 1) + (i - 1)] - tau[base - i];
+        const double* prev = row[(l - 1) & 1];   // tau_{base - i} = prev[k - i]
+        double* cur = row[l & 1];
+        const double g = next;
+        next = product(l + 1);
+        if (l >= 2 && i == 0) tau[base] = cur[0] = diag[k + l - 2];
+        if (i >= 1 && i < k && base + i < n_terms) tau[base + i] = cur[i] = 2.0 * g - prev[k - i];
         __syncthreads();
     }
 }
@@ -1126,7 +1135,7 @@ cudaError_t launch_set_io(const InstIO* ios, int count, InstIO* d_io, const Inst
         p.count = count - c0 < kIoChunk ? count - c0 : kIoChunk;
         p.first = first + c0;
         for (int j = 0; j < p.count; ++j) p.io[j] = ios[c0 + j];
-        launch_pdl(k_set_io, 1, kIoChunk, 0, s, p, d_io, d_inst);
+        launch_pdl(count, k_set_io, 1, kIoChunk, 0, s, p, d_io, d_inst);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1136,34 +1145,34 @@ cudaError_t launch_set_io(const InstIO* ios, int count, InstIO* d_io, const Inst
 cudaError_t launch_bounds(const Inst* in, const InstIO* io, int batch, Work wg, double* part,
                           int use_given, cudaStream_t s) {
     if (use_given) {
-        launch_pdl(k_bounds_given, (batch + 127) / 128, 128, 0, s, in, io, batch);
+        launch_pdl(batch, k_bounds_given, (batch + 127) / 128, 128, 0, s, in, io, batch);
         return cudaGetLastError();
     }
-    launch_pdl(k_gershgorin_rows, wg.total, 32 * kGershRows, 0, s, in, io, wg, part);
-    launch_pdl(k_gershgorin_final, batch, 256, 0, s, in, wg, part);
+    launch_pdl(batch, k_gershgorin_rows, wg.total, 32 * kGershRows, 0, s, in, io, wg, part);
+    launch_pdl(batch, k_gershgorin_final, batch, 256, 0, s, in, wg, part);
     return cudaGetLastError();
 }
 
 cudaError_t launch_export_bounds(const DevResult* res, double* out3, cudaStream_t s) {
-    launch_pdl(k_export_bounds, 1, 1, 0, s, res, out3);
+    launch_pdl(1, k_export_bounds, 1, 1, 0, s, res, out3);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scale(const Inst* in, const InstIO* io, Work ws, const Shape& sh, cudaStream_t s,
                          int* dbg) {
-    launch_pdl(k_scale_sym, ws.total, 256, 0, s, in, io, ws, sh, dbg);
+    launch_pdl(ws.count, k_scale_sym, ws.total, 256, 0, s, in, io, ws, sh, dbg);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack_f32(const float* A, int64_t n, int64_t lda, char* slot, int64_t np, int planes,
                             int fp16, float pscale, cudaStream_t s) {
-    launch_pdl(k_pack_f32, grid_for(np * np, 256), 256, 0, s, A, n, lda, slot, np, planes, fp16, pscale);
+    launch_pdl(1, k_pack_f32, grid_for(np * np, 256), 256, 0, s, A, n, lda, slot, np, planes, fp16, pscale);
     return cudaGetLastError();
 }
 
 cudaError_t launch_diag_sums(const Inst* in, int batch, int count, const Shape& sh, cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
-    launch_pdl(k_diag_sums, dim3(count, batch), 256, 0, s, in, sh.is64);
+    launch_pdl(batch, k_diag_sums, dim3(count, batch), 256, 0, s, in, sh.is64);
     return cudaGetLastError();
 }
 
@@ -1189,10 +1198,10 @@ cudaError_t launch_gram_shape(const Inst* in, int batch, Work wgr, int giant0, i
         const int threads = gram_threads(ngq * nbq, TPW);
         if (is64) {
             cudaFuncSetAttribute(k_gram<double, TG, TB, TPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            launch_pdl(k_gram<double, TG, TB, TPW>, wgr.total, threads, smem, s, in, wgr, giant0 + g, ng, baby0, nbaby);
+            launch_pdl(batch, k_gram<double, TG, TB, TPW>, wgr.total, threads, smem, s, in, wgr, giant0 + g, ng, baby0, nbaby);
         } else {
             cudaFuncSetAttribute(k_gram<float, TG, TB, TPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            launch_pdl(k_gram<float, TG, TB, TPW>, wgr.total, threads, smem, s, in, wgr, giant0 + g, ng, baby0, nbaby);
+            launch_pdl(batch, k_gram<float, TG, TB, TPW>, wgr.total, threads, smem, s, in, wgr, giant0 + g, ng, baby0, nbaby);
         }
         const int npairs = ng * nbaby;
         k_sum_partials<<<dim3(npairs, batch), 128, 0, s>>>(in, npairs, (out_g0 + g) * nbaby);
@@ -1306,7 +1315,7 @@ cudaError_t launch_gram_ring(const Inst* in, int batch, Work wgr, const GramGeom
             const int u0 = geom.pre_host[gr.i0], u1 = geom.pre_host[gr.i1];
             if (u1 <= u0) continue;
             const int grid = u1 - u0 < sm_count() ? u1 - u0 : sm_count();
-            launch_pdl(k_gram_ring<TG, TB>, grid, 32 * (ncons + 1), smem, s, maps, in, wgr, u0, u1, gr.b0, giant0 + g, ng,
+            launch_pdl(batch, k_gram_ring<TG, TB>, grid, 32 * (ncons + 1), smem, s, maps, in, wgr, u0, u1, gr.b0, giant0 + g, ng,
                                                                      baby0, nbaby, H, S, CPS, err);
             if (launches) *launches += 1;
         }
@@ -1345,7 +1354,7 @@ cudaError_t launch_gram(const Inst* in, int batch, Work wgr, int giant0, int ngi
 }
 
 cudaError_t launch_assemble_moments(const Inst* in, int batch, const Shape& sh, cudaStream_t s) {
-    launch_pdl(k_assemble_moments, batch, 64, 0, s, in, sh.k, sh.m, sh.n_terms);
+    launch_pdl(batch, k_assemble_moments, batch, 64, 0, s, in, sh.k, sh.m, sh.n_terms);
     return cudaGetLastError();
 }
 
@@ -1353,18 +1362,18 @@ cudaError_t launch_tile_trace(const Inst* in, const InstIO* io, int batch, const
                               int mode, cudaStream_t s) {
     // 256 threads per instance: the partials and the diagonal of P (one sector per entry) are
     // read by enough threads to keep the loads in flight
-    launch_pdl(k_tile_trace, batch, 256, 0, s, in, io, pre, part, mode);
+    launch_pdl(batch, k_tile_trace, batch, 256, 0, s, in, io, pre, part, mode);
     return cudaGetLastError();
 }
 
 cudaError_t launch_trace_frob(const Inst* in, const InstIO* io, Work we, double* part, cudaStream_t s) {
-    launch_pdl(k_trace_frob_part, we.total, 256, 0, s, in, io, we, part);
-    launch_pdl(k_trace_frob_final, we.count, 32, 0, s, in, we, part);
+    launch_pdl(we.count, k_trace_frob_part, we.total, 256, 0, s, in, io, we, part);
+    launch_pdl(we.count, k_trace_frob_final, we.count, 32, 0, s, in, we, part);
     return cudaGetLastError();
 }
 
 cudaError_t launch_copy_out(const Inst* in, const InstIO* io, Work we, const Shape& sh, cudaStream_t s) {
-    launch_pdl(k_copy_out, we.total, 256, 0, s, in, io, we, sh.n_tslots, sh.is64);
+    launch_pdl(we.count, k_copy_out, we.total, 256, 0, s, in, io, we, sh.n_tslots, sh.is64);
     return cudaGetLastError();
 }
 
