@@ -438,53 +438,78 @@ __global__ void __launch_bounds__(256) k_poly_width(const Inst* __restrict__ ins
 }
 
 // R_l = g_{0,l} I_n + sum_{i=1}^{k-1} g_{i,l} T_i for all l < m, float64. T_i is slot i-1,
-// R_l slot n_tslots + l. A block covers ew_rows(np) rows of one instance; outputs are
-// produced in groups of kGroup l's per pass over the T_i.
-constexpr int kGroup = 16;
+// R_l slot n_tslots + l. The float64 FMAs bound it (two lanes per clock and SM), so only the entries
+// on and above the diagonal are formed: a block takes a 32 x 32 block (bi, bj), bj >= bi, of one
+// instance, four entries per thread, kGroup l's per pass over the T_i, and writes each R_l on both
+// sides of the diagonal (through shared memory). 400 terms, float64: N = 256 0.56 ms and N = 2000
+// 5.5 ms when every entry of the square was formed, in blocks of 8192 (eight of them at N = 256).
+constexpr int kGroup = 20;
+constexpr int kCtRows = 4;   // rows of the block per thread
 
-__global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ insts, Work we, int k,
+__global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ insts, Work ws, int k,
                                                       int m, int n_tslots) {
     pdl_sync();
-    extern __shared__ double gsh[];
-    const int i = find_inst(we.pre, 0, we.count, blockIdx.x);
+    extern __shared__ double gsh[];   // g (k m), then the 32 x 33 transposition tile
+    double (*tile)[33] = reinterpret_cast<double (*)[33]>(gsh + k * m);
+    const int i = find_inst(ws.pre, 0, ws.count, blockIdx.x);
     const Inst& in = insts[i];
     if (!in.res->active) return;
     for (int q = threadIdx.x; q < k * m; q += blockDim.x) gsh[q] = in.g[q];
     __syncthreads();
     const int64_t np = in.np, n = in.n;
-    const int rows = ew_rows(np);
-    const int64_t r0 = (int64_t)(blockIdx.x - we.pre[i]) * rows;
-    const int64_t r1 = r0 + rows < np ? r0 + rows : np;
+    int bi, bj;
+    upper_tile(blockIdx.x - ws.pre[i], (int)(np / 32), bi, bj);
     const int64_t tstride = in.slot_bytes / 8;
-    const double* tbase = reinterpret_cast<const double*>(in.slots);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    // entries (r0 + 8 u, c) of the block, u < kCtRows
+    const int64_t r0 = (int64_t)bi * 32 + ty, c = (int64_t)bj * 32 + tx;
+    const double* tbase = reinterpret_cast<const double*>(in.slots) + r0 * np + c;
     double* rbase = reinterpret_cast<double*>(in.slots + n_tslots * in.slot_bytes);
     // bits of the largest |entry| of the last R, the scale of its digits
     const int last = (in.res->m_eff > 0 ? in.res->m_eff : m) - 1;
     unsigned long long mx = 0;
-    for (int64_t idx = r0 * np + threadIdx.x; idx < r1 * np; idx += blockDim.x) {
-        const int64_t r = idx / np, col = idx - r * np;
-        const bool diag = (r == col) && (r < n);
-        for (int l0 = 0; l0 < m; l0 += kGroup) {
-            double acc[kGroup];
+    for (int l0 = 0; l0 < m; l0 += kGroup) {
+        double acc[kGroup][kCtRows];
 #pragma unroll
-            for (int q = 0; q < kGroup; ++q) acc[q] = 0.0;
-            for (int t = 1; t < k; ++t) {
-                const double v = tbase[(int64_t)(t - 1) * tstride + idx];
+        for (int q = 0; q < kGroup; ++q)
 #pragma unroll
-                for (int q = 0; q < kGroup; ++q)
-                    if (l0 + q < m) acc[q] = fma(gsh[(l0 + q) * k + t], v, acc[q]);
-            }
+            for (int u = 0; u < kCtRows; ++u) acc[q][u] = 0.0;
+#pragma unroll 1
+        for (int t = 1; t < k; ++t) {
+            double v[kCtRows];
+#pragma unroll
+            for (int u = 0; u < kCtRows; ++u) v[u] = __ldg(tbase + (int64_t)(t - 1) * tstride + (int64_t)(8 * u) * np);
 #pragma unroll
             for (int q = 0; q < kGroup; ++q) {
-                if (l0 + q < m) {
-                    double v = acc[q];
-                    if (diag) v += gsh[(l0 + q) * k];
-                    rbase[(int64_t)(l0 + q) * tstride + idx] = v;
+                const double g = l0 + q < m ? gsh[(l0 + q) * k + t] : 0.0;
+#pragma unroll
+                for (int u = 0; u < kCtRows; ++u) acc[q][u] = fma(g, v[u], acc[q][u]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kGroup; ++q) {
+            if (l0 + q >= m) break;
+            double* R = rbase + (int64_t)(l0 + q) * tstride;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < kCtRows; ++u) {
+                const int64_t r = r0 + 8 * u;
+                double v = acc[q][u];
+                if (r == c && r < n) v += gsh[(l0 + q) * k];
+                tile[ty + 8 * u][tx] = v;
+                if (bi != bj || c >= r) {   // a diagonal block's lower half mirrors its upper half
+                    R[r * np + c] = v;
                     if (l0 + q == last) {
                         const unsigned long long av = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
                         mx = av > mx ? av : mx;
                     }
                 }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < kCtRows; ++u) {
+                const int64_t r = (int64_t)bj * 32 + ty + 8 * u, cc = (int64_t)bi * 32 + tx;
+                if (bi != bj || cc < r) R[r * np + cc] = tile[tx][ty + 8 * u];
             }
         }
     }
@@ -782,10 +807,10 @@ cudaError_t launch_g_to_d(const Inst* in, int batch, const Shape& sh, cudaStream
 
 cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const Shape& sh, cudaStream_t s, int* dbg) {
     if (sh.is64) {
-        const size_t smem = (size_t)sh.k * sh.m * sizeof(double);
+        const size_t smem = ((size_t)sh.k * sh.m + 32 * 33) * sizeof(double);
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_contract_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(we.count, k_contract_f64, we.total, 256, smem, s, in, we, sh.k, sh.m, sh.n_tslots);
+        launch_pdl(wsym.count, k_contract_f64, wsym.total, 256, smem, s, in, wsym, sh.k, sh.m, sh.n_tslots);
         return cudaGetLastError();
     }
     const int planes_last = sh.m > 1 ? sh.planes : 0;

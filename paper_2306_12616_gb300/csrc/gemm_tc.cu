@@ -846,8 +846,11 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     constexpr int RPW = kBM / DW;          // tile rows per drain warp
     constexpr int HPR = TBN / 64;          // 64-column pieces per row
     constexpr int NIT = RPW * HPR;
-    constexpr int G = DW == 16 ? 4 : 8;    // 16 drain warps run at the 96-register cap
+    // two iterations at a time: this code runs once or twice per call, so its instructions come from
+    // memory; eight unrolled took 46 us for one tile at N = 64
+    constexpr int G = 2;
     static_assert(NIT % G == 0, "row-pass groups");
+#pragma unroll 1
     for (int q0 = 0; q0 < NIT; q0 += G) {
         float2 cv[G], dv[G];
 #pragma unroll
@@ -955,6 +958,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     asm volatile("bar.sync 1, %0;" ::"n"(32 * DW) : "memory");
     // mirror pass: output row n0 + c holds tile column c for the entries with col > row;
     // each drain warp takes TBN / 8 tile columns, lanes on row pairs
+#pragma unroll 1
     for (int cc = 0; cc < TBN / DW; ++cc) {
         const int c = ew * (TBN / DW) + cc;
         const int64_t grow = (int64_t)n0 + c;       // output row

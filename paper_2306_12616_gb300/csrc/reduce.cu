@@ -420,6 +420,15 @@ __host__ __device__ inline int64_t upper_chunks(int64_t np, int kc) {
     return (int64_t)kc * cpr * (cpr + 1) / 2;
 }
 
+// Chunks per block. float32: kGChunks (the partial sums' grouping is part of the result's bits).
+// float64: as few as give an instance about 300 blocks, since the float64 FMAs bound the kernel and a
+// small matrix would otherwise use few SMs (N = 256: 10 blocks of 64 chunks, 0.35 ms).
+__host__ __device__ inline int gram_chunks(int64_t np, bool is64) {
+    if (!is64) return kGChunks;
+    const int64_t c = upper_chunks(np, kChunkBytes / 8) / 300;
+    return c < 2 ? 2 : (c > kGChunks ? kGChunks : (int)c);
+}
+
 template <typename T, int TG, int TB, int TPW>
 __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const Inst* __restrict__ insts, Work wgr, int giant0,
                                                           int ngiant, int baby0, int nbaby) {
@@ -439,8 +448,9 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const Inst* __restrict
     const int64_t np = in.np;
     const int64_t cpr = np / kChunk;                  // chunks per row
     const int64_t nchunks = upper_chunks(np, kChunk);
-    const int64_t c0 = (int64_t)lb * kGChunks;
-    const int64_t c1 = c0 + kGChunks < nchunks ? c0 + kGChunks : nchunks;
+    const int per = gram_chunks(np, sizeof(T) == 8);
+    const int64_t c0 = (int64_t)lb * per;
+    const int64_t c1 = c0 + per < nchunks ? c0 + per : nchunks;
     const int ngq = (ngiant + TG - 1) / TG, nbq = (nbaby + TB - 1) / TB;
     const int nrows = TG * ngq + TB * nbq;
     const int ntiles = ngq * nbq;
@@ -1178,7 +1188,8 @@ cudaError_t launch_diag_sums(const Inst* in, int batch, int count, const Shape& 
 
 int gram_blocks_for(int64_t np, int is64) {
     const int64_t u = upper_chunks(np, kChunkBytes / (is64 ? 8 : 4));
-    return (int)((u + kGChunks - 1) / kGChunks);
+    const int per = gram_chunks(np, is64 != 0);
+    return (int)((u + per - 1) / per);
 }
 
 template <int TG, int TB, int TPW>
