@@ -60,7 +60,8 @@ struct Group {           // instances [i0, i1) with buckets [b0, b0 + nb): one g
 
 struct HostWork {
     std::vector<int> pre;
-    Work dev{nullptr, 0, 0};
+    std::vector<int> tab;       // instance of every block (batches of more than a few instances)
+    Work dev{nullptr, 0, 0, nullptr};
 };
 
 struct Plan {
@@ -85,6 +86,8 @@ struct Plan {
     HostWork wg, wsc, we, wr, wgr, wct, wtc[2], wf64;   // wtc[0]: 256-wide tiles, wtc[1]: 128-wide
     bool digits = false;      // float64 products on the tensor cores (gemm_digits.cu)
     HostWork wdig;            // their units
+    std::vector<uint2> ttab[2];   // split products: (instance, row block << 16 | column tile) per tile
+    const uint2* d_ttab[2] = {nullptr, nullptr};
     std::vector<unsigned char> dig_maps;   // 128 bytes per bucket
     int tile_n = 0;
     int tile_ctas = 0;
@@ -434,6 +437,9 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     auto fill = [&](HostWork& w, auto count) {
         w.pre.assign(batch + 1, 0);
         for (int j = 0; j < batch; ++j) w.pre[j + 1] = w.pre[j] + (int)count(p->inst[j]);
+        w.tab.clear();
+        if (batch > kSmallBatch)
+            for (int j = 0; j < batch; ++j) w.tab.insert(w.tab.end(), w.pre[j + 1] - w.pre[j], j);
     };
     fill(p->wg, [](const Inst& in) { return (in.n + kGershRows - 1) / kGershRows; });
     fill(p->wsc, [](const Inst& in) { const int64_t t = in.np / 32; return t * (t + 1) / 2; });
@@ -444,6 +450,18 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     const bool full = key.mode == MODE_PRODUCT && !key.sym;
     fill(p->wtc[0], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 256) : tc_tiles(in.np, 256); });
     fill(p->wtc[1], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 128) : tc_tiles(in.np, 128); });
+    for (int q = 0; q < 2 && !sh.is64; ++q) {
+        // the tiles of the two work lists, in their order: row blocks, and within them the column
+        // tiles that reach the diagonal (all of them for a product that is not symmetric)
+        const int width = q == 0 ? 256 : 128;
+        p->ttab[q].reserve((size_t)p->wtc[q].pre[batch]);
+        for (int j = 0; j < batch; ++j) {
+            const int tm = (int)(p->inst[j].np / kPad), tn = (int)((p->inst[j].np + width - 1) / width);
+            for (int I = 0; I < tm; ++I)
+                for (int J = full ? 0 : I * kPad / width; J < tn; ++J)
+                    p->ttab[q].push_back(make_uint2((unsigned)j, ((unsigned)I << 16) | (unsigned)J));
+        }
+    }
     fill(p->wf64, [](const Inst& in) { return f64_tiles(in.np); });
     fill(p->wdig, [&](const Inst& in) { return p->digits ? dig_units(in.np, in.dig_sl, in.dig_sh) : int64_t(0); });
     const size_t off_pg = take(8 * 3 * (size_t)std::max(1, p->wg.pre[batch]));
@@ -522,7 +540,8 @@ fo_status place_plan(fo_ctx* ctx, Plan* p) {
     HostWork* lists[] = {&p->wg,  &p->wsc,    &p->we,     &p->wr,   &p->wgr,
                          &p->wct, &p->wtc[0], &p->wtc[1], &p->wf64, &p->wdig};
     size_t bytes = align256(sizeof(Inst) * batch) + align256(sizeof(InstIO) * batch);
-    for (HostWork* w : lists) bytes += align256(sizeof(int) * w->pre.size());
+    for (HostWork* w : lists) bytes += align256(sizeof(int) * w->pre.size()) + align256(sizeof(int) * w->tab.size());
+    for (const auto& t : p->ttab) bytes += align256(sizeof(uint2) * t.size());
     const size_t off_ct = bytes;
     bytes += align256(8 * 4 * (size_t)sh.M);
     if (cudaMalloc(&p->dtab, bytes) != cudaSuccess) {
@@ -543,6 +562,18 @@ fo_status place_plan(fo_ctx* ctx, Plan* p) {
         w->dev.total = w->pre[batch];
         std::memcpy(host.data() + o, w->pre.data(), sizeof(int) * w->pre.size());
         o += align256(sizeof(int) * w->pre.size());
+        w->dev.tab = nullptr;
+        if (!w->tab.empty()) {
+            w->dev.tab = reinterpret_cast<const int*>(reinterpret_cast<char*>(p->dtab) + o);
+            std::memcpy(host.data() + o, w->tab.data(), sizeof(int) * w->tab.size());
+            o += align256(sizeof(int) * w->tab.size());
+        }
+    }
+    for (int q = 0; q < 2; ++q) {
+        p->d_ttab[q] = reinterpret_cast<const uint2*>(reinterpret_cast<char*>(p->dtab) + o);
+        if (!p->ttab[q].empty()) std::memcpy(host.data() + o, p->ttab[q].data(), sizeof(uint2) * p->ttab[q].size());
+        o += align256(sizeof(uint2) * p->ttab[q].size());
+        p->ttab[q] = std::vector<uint2>();   // only the device copy is used
     }
     if (cudaMemcpy(p->dtab, host.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(ctx, FO_ERR_CUDA, "plan table upload failed");
@@ -657,7 +688,8 @@ fo_status run_products(fo_ctx* ctx, Plan& p, const Step* steps, int nsteps, cuda
                 std::string err;
                 const int tile0 = w.pre[g.i0];
                 cudaError_t e = tc_gemm(prec, p.tile_n, p.tile_ctas, p.tile_drain, steps + q0, nq, p.d_inst, p.d_io,
-                                        w.dev.pre, g.i0, g.i1, tile0, w.pre[g.i1] - tile0,
+                                        w.dev.pre, p.d_ttab[p.tile_n == 128 ? 1 : 0], g.i0, g.i1, tile0,
+                                        w.pre[g.i1] - tile0,
                                         p.maps.data() + 256 * (size_t)g.b0, g.b0, g.nb, ctx->flag, s, &err,
                                         p.key.sym ? (p.sh.ublk ? 2 : 1) : 0, p.tile_persist);
                 if (e == cudaSuccess && debug_sync() && !ctx->capturing) e = cudaDeviceSynchronize();

@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ i
     pdl_sync();
     extern __shared__ double gsh[];   // g (k m), then the 32 x 33 transposition tile
     double (*tile)[33] = reinterpret_cast<double (*)[33]>(gsh + k * m);
-    const int i = find_inst(ws.pre, 0, ws.count, blockIdx.x);
+    const int i = inst_of(ws, blockIdx.x);
     const Inst& in = insts[i];
     if (!in.res->active) return;
     for (int q = threadIdx.x; q < k * m; q += blockDim.x) gsh[q] = in.g[q];
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(128, 4) k_contract_f32(const Inst* __restrict_
     static_assert(MAXM % 4 == 0, "l pairs per half");
     constexpr int HM = MAXM / 2;                           // R_l per thread
     extern __shared__ __align__(16) float fsh[];
-    const int i = find_inst(wct.pre, 0, wct.count, blockIdx.x);
+    const int i = inst_of(wct, blockIdx.x);
     const Inst& in = insts[i];
     if (!in.res->active) return;
     const int tid = threadIdx.x;
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(256) k_mirror_planes(const Inst* __restrict__ 
                                                        int planes, int ublk, int* dbg) {
     pdl_sync();
     __shared__ uint16_t tile[3][32][33];
-    const int i = find_inst(ws.pre, 0, ws.count, blockIdx.x);
+    const int i = inst_of(ws, blockIdx.x);
     if (!insts[i].res->active) return;
     // the instance's last R: R_{m-1}, or R_{m_eff-1} for an expansion cut by a learned order
     const int slot = slot0 + (insts[i].res->m_eff > 0 ? insts[i].res->m_eff : m) - 1;

@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __r
     __shared__ double sv[32][33];
     __shared__ unsigned long long su[32][33];
     __shared__ int s_e[2];
-    const int inst = find_inst(ws.pre, 0, ws.count, blockIdx.x);
+    const int inst = inst_of(ws, blockIdx.x);
     const Inst& in = insts[inst];
     if (!step_needed(in.res, st.need_m)) return;
     const int64_t n = in.n, np = in.np;
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __r
 __global__ void __launch_bounds__(128) k_dig_split(const Inst* __restrict__ insts, Work ws, int slot0, int last_m,
                                                    int buf, int need_m) {
     pdl_sync();
-    const int inst = find_inst(ws.pre, 0, ws.count, blockIdx.x);
+    const int inst = inst_of(ws, blockIdx.x);
     const Inst& in = insts[inst];
     if (!step_needed(in.res, need_m)) return;
     const int slot = last_m > 0 ? slot0 + (in.res->m_eff > 0 ? in.res->m_eff : last_m) - 1 : slot0;

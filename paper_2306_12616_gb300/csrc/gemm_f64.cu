@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(256) k_gemm_f64(const __grid_constant__ StepLi
     const int sidx = blockIdx.x / wt.total;
     const int bt = blockIdx.x - sidx * wt.total;
     const Step& st = steps.s[sidx];
-    const int inst = find_inst(wt.pre, 0, wt.count, bt);
+    const int inst = inst_of(wt, bt);
     const Inst& in = insts[inst];
     if (!step_needed(in.res, st.need_m)) return;
     const int64_t np = in.np;

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     k_tc_gemm(const __grid_constant__ TcMaps maps,
               const __grid_constant__ std::conditional_t<CHAIN, ChainList, StepList> steps,
               const Inst* __restrict__ insts, const InstIO* __restrict__ io, const int* __restrict__ pre,
-              int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag) {
+              const uint2* __restrict__ tab, int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag) {
     using Cfg = TcCfg<PA, PB, NPROD, F16, TBN, MINB, DW>;
     constexpr int S = Cfg::kStages;
     constexpr int NC = Cfg::kCols;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
 
     if constexpr (!CHAIN) pdl_launch();
     // ---------------- step, instance and tile of this CTA (uniform across the CTA)
-    int sidx, gtile, inst;
+    int sidx, gtile, inst, I, J;
     // chain launches: the ticket's step and the tile count its instance must reach first,
     // kept in shared memory (re-read after the main loop instead of held in registers)
     __shared__ int s_chain[4];   // ticket, step, count needed, stop
@@ -280,7 +280,10 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     } else {
         sidx = (int)blockIdx.x / tiles;
         gtile = tile0 + (int)blockIdx.x - sidx * tiles;
-        inst = find_inst(pre, i0, i1, gtile);
+        const uint2 e = __ldg(tab + gtile);
+        inst = (int)e.x;
+        I = (int)(e.y >> 16);
+        J = (int)(e.y & 0xffffu);
     }
     const Step& st = steps.s[sidx];
     const Inst& in = insts[inst];
@@ -300,9 +303,7 @@ __global__ void __launch_bounds__(32 * (2 + DW), MINB)
 
     // the warp index through a shuffle: a role's branch is then known to be uniform
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int tm = np / kBM, tn = (np + TBN - 1) / TBN;
-    int I, J;
-    tile_of(gtile - __ldg(pre + inst), tm, tn, TBN, sym, I, J);
+    if constexpr (CHAIN) tile_of(gtile - __ldg(pre + inst), np / kBM, (np + TBN - 1) / TBN, TBN, sym, I, J);
     const int m0 = I * kBM;
     int n0 = J * TBN;
     // k-blocks. The zero border past column n contributes exact zeros, so 128-wide tiles stop
@@ -1563,32 +1564,32 @@ EncodeFn get_encode(std::string* err) {
 
 template <int PA, int PB, int NPROD, bool F16, int TBN, int MINB, int DW, bool CHAIN, class SL>
 cudaError_t launch_tc(const TcMaps& maps, const SL& st, unsigned grid, const Inst* in, const InstIO* io,
-                      const int* pre, int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag,
+                      const int* pre, const uint2* tab, int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag,
                       cudaStream_t s) {
     using Cfg = TcCfg<PA, PB, NPROD, F16, TBN, MINB, DW>;
     auto kern = k_tc_gemm<PA, PB, NPROD, F16, TBN, MINB, DW, CHAIN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
     if (e != cudaSuccess) return e;
     if constexpr (!CHAIN)
-        return launch_pdl(kern, grid, Cfg::kThreads, Cfg::kSmem, s, maps, st, in, io, pre, i0, i1, tile0, tiles, b0,
-                          sym, err_flag);
-    kern<<<grid, Cfg::kThreads, Cfg::kSmem, s>>>(maps, st, in, io, pre, i0, i1, tile0, tiles, b0, sym, err_flag);
+        return launch_pdl(kern, grid, Cfg::kThreads, Cfg::kSmem, s, maps, st, in, io, pre, tab, i0, i1, tile0, tiles,
+                          b0, sym, err_flag);
+    kern<<<grid, Cfg::kThreads, Cfg::kSmem, s>>>(maps, st, in, io, pre, tab, i0, i1, tile0, tiles, b0, sym, err_flag);
     return cudaGetLastError();
 }
 
 template <int PA, int PB, int NPROD, bool F16, bool CHAIN, class SL>
 cudaError_t dispatch_tbn(int tile_n, int ctas, int drain, const TcMaps& maps, const SL& st, unsigned grid,
-                         const Inst* in, const InstIO* io, const int* pre, int i0, int i1, int tile0, int tiles,
+                         const Inst* in, const InstIO* io, const int* pre, const uint2* tab, int i0, int i1, int tile0, int tiles,
                          int b0, int sym, int* err_flag, cudaStream_t s) {
     if (tile_n == 256)
-        return drain == 16 ? launch_tc<PA, PB, NPROD, F16, 256, 1, 16, CHAIN>(maps, st, grid, in, io, pre, i0, i1,
+        return drain == 16 ? launch_tc<PA, PB, NPROD, F16, 256, 1, 16, CHAIN>(maps, st, grid, in, io, pre, tab, i0, i1,
                                                                                tile0, tiles, b0, sym, err_flag, s)
-                           : launch_tc<PA, PB, NPROD, F16, 256, 1, 8, CHAIN>(maps, st, grid, in, io, pre, i0, i1,
+                           : launch_tc<PA, PB, NPROD, F16, 256, 1, 8, CHAIN>(maps, st, grid, in, io, pre, tab, i0, i1,
                                                                               tile0, tiles, b0, sym, err_flag, s);
     if (ctas == 2)
-        return launch_tc<PA, PB, NPROD, F16, 128, 2, 8, CHAIN>(maps, st, grid, in, io, pre, i0, i1, tile0, tiles, b0,
+        return launch_tc<PA, PB, NPROD, F16, 128, 2, 8, CHAIN>(maps, st, grid, in, io, pre, tab, i0, i1, tile0, tiles, b0,
                                                                sym, err_flag, s);
-    return launch_tc<PA, PB, NPROD, F16, 128, 1, 8, CHAIN>(maps, st, grid, in, io, pre, i0, i1, tile0, tiles, b0, sym,
+    return launch_tc<PA, PB, NPROD, F16, 128, 1, 8, CHAIN>(maps, st, grid, in, io, pre, tab, i0, i1, tile0, tiles, b0, sym,
                                                            err_flag, s);
 }
 
@@ -1613,17 +1614,17 @@ cudaError_t launch_persist(const TcMaps& maps, const StepList& st, const Inst* i
 
 template <bool CHAIN, class SL>
 cudaError_t dispatch_prec(int prec, int tile_n, int ctas, int drain, const TcMaps& maps, const SL& st, unsigned grid,
-                          const Inst* in, const InstIO* io, const int* pre, int i0, int i1, int tile0, int tiles,
+                          const Inst* in, const InstIO* io, const int* pre, const uint2* tab, int i0, int i1, int tile0, int tiles,
                           int b0, int sym, int* err_flag, cudaStream_t s) {
     switch (prec) {
         case FO_PREC_BF16X3:
-            return dispatch_tbn<3, 3, 6, false, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, i0, i1,
+            return dispatch_tbn<3, 3, 6, false, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, tab, i0, i1,
                                                        tile0, tiles, b0, sym, err_flag, s);
         case FO_PREC_FP16X2:
-            return dispatch_tbn<2, 2, 3, true, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, i0, i1,
+            return dispatch_tbn<2, 2, 3, true, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, tab, i0, i1,
                                                       tile0, tiles, b0, sym, err_flag, s);
         case FO_PREC_BF16X1:
-            return dispatch_tbn<1, 1, 1, false, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, i0, i1,
+            return dispatch_tbn<1, 1, 1, false, CHAIN>(tile_n, ctas, drain, maps, st, grid, in, io, pre, tab, i0, i1,
                                                        tile0, tiles, b0, sym, err_flag, s);
         default: return cudaErrorInvalidValue;
     }
@@ -1719,8 +1720,9 @@ bool gram_make_map(void* map128, const GramBucket& b, int nslots, int box_slots,
 }
 
 cudaError_t tc_gemm(int prec, int tile_n, int ctas, int drain, const Step* steps, int nsteps, const Inst* in,
-                    const InstIO* io, const int* pre, int i0, int i1, int tile0, int tiles, const void* maps, int b0,
-                    int nb, int* err_flag, cudaStream_t s, std::string* err, int sym, int persist) {
+                    const InstIO* io, const int* pre, const uint2* tab, int i0, int i1, int tile0, int tiles,
+                    const void* maps, int b0, int nb, int* err_flag, cudaStream_t s, std::string* err, int sym,
+                    int persist) {
     if (!tile_config_ok(prec, tile_n, ctas, drain) || nb < 1 || nb > kMaxBuckets || !err_flag || nsteps < 1 ||
         nsteps > kMaxSteps || (persist && tile_n != 128)) {
         if (err) *err = "tc_gemm: unsupported precision, tile or bucket count";
@@ -1743,7 +1745,7 @@ cudaError_t tc_gemm(int prec, int tile_n, int ctas, int drain, const Step* steps
             default: return cudaErrorInvalidValue;
         }
     }
-    return dispatch_prec<false>(prec, tile_n, ctas, drain, tm, st, (unsigned)(tiles * nsteps), in, io, pre, i0, i1,
+    return dispatch_prec<false>(prec, tile_n, ctas, drain, tm, st, (unsigned)(tiles * nsteps), in, io, pre, tab, i0, i1,
                                 tile0, tiles, b0, sym, err_flag, s);
 }
 
@@ -1791,7 +1793,7 @@ cudaError_t tc_chain(int prec, int tile_n, int ctas, int drain, const Step* step
     if (e != cudaSuccess) return e;
     TcMaps tm;
     copy_maps(tm, maps, nb);
-    return dispatch_prec<true>(prec, tile_n, ctas, drain, tm, cl, (unsigned)base, in, io, pre_dev, i0, i1, 0, 0, b0,
+    return dispatch_prec<true>(prec, tile_n, ctas, drain, tm, cl, (unsigned)base, in, io, pre_dev, nullptr, i0, i1, 0, 0, b0,
                                sym, err_flag, s);
 }
 

@@ -152,10 +152,13 @@ struct ChainList {
 };
 
 // The block-to-instance map of a grouped launch: pre[j] = blocks of instances < j.
+// A batch of more than a few instances also has the map itself (tab[b] = instance of block b): a
+// binary search over 512 instances is nine dependent loads, 2000 clocks at the head of every block.
 struct Work {
     const int* pre;   // device, count + 1 entries
     int count;        // instances
     int total;        // blocks
+    const int* tab;   // device, total entries, or null
 };
 
 // Programmatic dependent launch. The kernels of a call form a chain on one stream; launched
@@ -219,6 +222,11 @@ __device__ __forceinline__ int find_inst(const int* __restrict__ pre, int lo, in
         else hi = mid;
     }
     return lo;
+}
+
+// The instance of block b of a grouped launch.
+__device__ __forceinline__ int inst_of(const Work& w, int b) {
+    return w.tab ? __ldg(w.tab + b) : find_inst(w.pre, 0, w.count, b);
 }
 
 // Tile (bi, bj), bj >= bi, that is the b-th of the upper triangle of a tn x tn tile grid in
@@ -569,11 +577,12 @@ bool tc_make_map(void* map128, const void* planes0, int64_t np, int nplanes, int
 // ctas = CTAs per SM (2 only with tile_n = 128). sym = 0 computes every tile of the full
 // product (fo_recurrence_product only), 1 the tiles on and above the diagonal of a symmetric
 // product over fully stored planes, 2 the same over planes stored as upper 128-blocks.
-// drain = TMEM drain warps (8, or 16 with 256-wide tiles).
+// drain = TMEM drain warps (8, or 16 with 256-wide tiles). tab: per tile of the work list its
+// (instance, row block << 16 | column tile).
 // persist = 1: the persistent kernel (tile_n = 128; one CTA per SM walks the tiles, with
 // separate epilogue warps overlapping each tile's epilogue with the next tile's products).
 cudaError_t tc_gemm(int prec, int tile_n, int ctas, int drain, const Step* steps, int nsteps, const Inst* in, const InstIO* io,
-                    const int* pre, int i0, int i1, int tile0, int tiles, const void* maps, int b0,
+                    const int* pre, const uint2* tab, int i0, int i1, int tile0, int tiles, const void* maps, int b0,
                     int nb, int* err_flag, cudaStream_t s, std::string* err, int sym = 1, int persist = 0);
 // A chain of dependent symmetric products (ChainList) over instances [i0, i1) in one launch,
 // windows of consecutive instances holding at least `win_tiles` tiles per step each (0: one

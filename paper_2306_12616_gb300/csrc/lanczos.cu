@@ -23,6 +23,7 @@ constexpr uint64_t kLzSeed = 0x4C414E43ull;
 constexpr double kLzMargin = 0.01;
 constexpr int kLzLoads = 16;    // columns per lane in flight (matrix-vector product)
 constexpr int kLzCluster = 8;   // one-warp blocks per instance of the update
+constexpr int kLzKeep = 8;      // rows per thread of the update kept in registers
 
 __device__ __forceinline__ double warp_sum_d(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(32 * kGershRows) k_lz_matvec(const Inst* __res
     pdl_sync();
     __shared__ double sp[kGershRows];
     const int b = blockIdx.x;
-    const int i = find_inst(wg.pre, 0, wg.count, b);
+    const int i = inst_of(wg, b);
     const Inst& in = insts[i];
     const Lz z = lz_of(in);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -159,6 +160,14 @@ __global__ void __cluster_dims__(kLzCluster, 1, 1) __launch_bounds__(32)
     const int64_t n = in.n;
     const double bj = z.beta[j];
     const int p0 = wg.pre[i], p1 = wg.pre[i + 1];
+    // up to kLzKeep of this thread's rows stay in registers, requested before the sum of the partials
+    double wk[kLzKeep], qk[kLzKeep];
+#pragma unroll
+    for (int u = 0; u < kLzKeep; ++u) {
+        const int64_t r = w * 32 + lane + (int64_t)u * 32 * kLzCluster;
+        wk[u] = r < n ? z.w[r] : 0.0;
+        qk[u] = r < n ? z.q[r] : 0.0;
+    }
     double a = 0.0;
     for (int c0 = p0; c0 < p1; c0 += kChunk) {
         const int m = p1 - c0 < kChunk ? p1 - c0 : kChunk;
@@ -169,7 +178,14 @@ __global__ void __cluster_dims__(kLzCluster, 1, 1) __launch_bounds__(32)
         __syncwarp();
     }
     double s = 0.0;
-    for (int64_t r = w * 32 + lane; r < n; r += 32 * kLzCluster) {
+#pragma unroll
+    for (int u = 0; u < kLzKeep; ++u) {
+        if (w * 32 + lane + (int64_t)u * 32 * kLzCluster >= n) break;
+        wk[u] = wk[u] - a * qk[u];
+        s = fma(wk[u], wk[u], s);
+    }
+    const int64_t rest = w * 32 + lane + (int64_t)kLzKeep * 32 * kLzCluster;
+    for (int64_t r = rest; r < n; r += 32 * kLzCluster) {
         const double wv = z.w[r] - a * z.q[r];
         z.w[r] = wv;
         s = fma(wv, wv, s);
@@ -180,9 +196,18 @@ __global__ void __cluster_dims__(kLzCluster, 1, 1) __launch_bounds__(32)
     const double bnext = sqrt(warp_sum_d(lane < kLzCluster ? sh[lane] : 0.0));
     // an invariant subspace, or n steps (the whole space)
     const bool stop = !(bnext > 1e-12 * (fabs(a) + bj)) || j + 1 >= n;
-    for (int64_t r = w * 32 + lane; r < n && !stop; r += 32 * kLzCluster) {
-        z.qp[r] = z.q[r];
-        z.q[r] = z.w[r] / bnext;
+    if (!stop) {
+#pragma unroll
+        for (int u = 0; u < kLzKeep; ++u) {
+            const int64_t r = w * 32 + lane + (int64_t)u * 32 * kLzCluster;
+            if (r >= n) break;
+            z.qp[r] = qk[u];
+            z.q[r] = wk[u] / bnext;
+        }
+        for (int64_t r = rest; r < n; r += 32 * kLzCluster) {
+            z.qp[r] = z.q[r];
+            z.q[r] = z.w[r] / bnext;
+        }
     }
     cl.sync();   // every block has read the record before it changes, and left the shared sums
     if (w == 0 && lane == 0) {

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(32 * kGershRows) k_gershgorin_rows(const Inst*
                                                                      Work wg, double* part) {
     pdl_sync();
     const int b = blockIdx.x;
-    const int i = find_inst(wg.pre, 0, wg.count, b);
+    const int i = inst_of(wg, b);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = insts[i].n, ld = io[i].ldh;
     const double* H = io[i].H;
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ inst
     pdl_sync();
     __shared__ double tile[32][33];
     __shared__ float tf[32][33];
-    const int i = find_inst(ws.pre, 0, ws.count, blockIdx.x);
+    const int i = inst_of(ws, blockIdx.x);
     const int64_t n = insts[i].n, np = insts[i].np, ld = io[i].ldh;
     const double* H = io[i].H;
     const DevResult* res = insts[i].res;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const Inst* __restrict
     constexpr int V = 16 / sizeof(T);          // elements per 16-byte vector
     constexpr int RS = kChunk + V;             // row stride (elements)
     constexpr int VPR = kChunk / V;            // vectors per row
-    const int i = find_inst(wgr.pre, 0, wgr.count, blockIdx.x);
+    const int i = inst_of(wgr, blockIdx.x);
     const Inst& in = insts[i];
     if (!in.res->active) return;
     const int lb = blockIdx.x - wgr.pre[i];
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
         int64_t issued = 0;                 // stages whose copies were issued
         bool stop = false;
         for (int u = u0 + blockIdx.x; u < u1 && !stop; u += gridDim.x) {
-            const int i = find_inst(wgr.pre, 0, wgr.count, u);
+            const int i = inst_of(wgr, u);
             const Inst& in = insts[i];
             if (!in.res->active) continue;
             const int64_t np = in.np, nchunks = upper_chunks(np, kRChunk);
@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
 #pragma unroll
         for (int b = 0; b < TB; ++b) acc[a][b] = make_float2(0.0f, 0.0f);
     for (int u = u0 + blockIdx.x; u < u1; u += gridDim.x) {
-        const int i = find_inst(wgr.pre, 0, wgr.count, u);
+        const int i = inst_of(wgr, u);
         const Inst& in = insts[i];
         if (!in.res->active) continue;
         const int64_t nchunks = upper_chunks(in.np, kRChunk);
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(256) k_trace_frob_part(const Inst* __restrict_
                                                          double* partials) {
     pdl_sync();
     __shared__ double sh[33];
-    const int i = find_inst(we.pre, 0, we.count, blockIdx.x);
+    const int i = inst_of(we, blockIdx.x);
     const int64_t n = insts[i].n, np = insts[i].np, ldp = io[i].ldp;
     const double* P = io[i].P;
     const int rows = red_rows(np);
@@ -1110,7 +1110,7 @@ __global__ void k_tile_trace(const Inst* __restrict__ insts, const InstIO* __res
 __global__ void k_copy_out(const Inst* __restrict__ insts, const InstIO* __restrict__ io, Work we,
                            int slot, int is64) {
     pdl_sync();
-    const int i = find_inst(we.pre, 0, we.count, blockIdx.x);
+    const int i = inst_of(we, blockIdx.x);
     if (!insts[i].res->active) return;
     const int64_t n = insts[i].n, np = insts[i].np, ldp = io[i].ldp;
     const int rows = ew_rows(np);
