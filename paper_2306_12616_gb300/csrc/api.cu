@@ -1095,7 +1095,10 @@ fo_status run_density(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run) {
 // on this plan's first baby step, timed with CUDA events on the plan's own layout (the data
 // are whatever the workspace holds; the work does not depend on them).
 fo_status autotune(fo_ctx* ctx, Plan& p) {
-    constexpr int kTuneReps = 5;   // timed products per candidate (the storages differ by a few per cent)
+    // timed products per candidate: the candidates differ by a few per cent, and short products are
+    // timed over about a millisecond (five of 30 us picked a tile 20 % slower on some runs)
+    constexpr int kTuneReps = 5, kTuneMost = 40;
+    constexpr float kTuneMs = 1.0f;
     p.sh.ublk = 0;
     if (p.sh.is64 || p.n_slots == 0) {
         p.tile_n = p.tile_ctas = p.tile_drain = p.tile_store = 0;
@@ -1122,7 +1125,8 @@ fo_status autotune(fo_ctx* ctx, Plan& p) {
     std::memset(io.data(), 0, sizeof(InstIO) * io.size());
     cudaStream_t s = nullptr;
     FO_CUDA(launch_set_io(io.data(), p.batch, p.d_io, p.d_inst, 0, s), "autotune setup");
-    const Step st = make_step(p, 0, 0, -1, -1, 1, 2.0, 0.0, -1.0, false, false, false, false, ctx);
+    // a recurrence step: out = 2 A B - C (slot 2, or the output's own slot, as C)
+    const Step st = make_step(p, 0, 0, p.n_slots > 2 ? 2 : 1, -1, 1, 2.0, -1.0, 0.0, false, false, false, false, ctx);
     cudaEvent_t e0 = ev_get(ctx), e1 = ev_get(ctx);
     float best = 0.0f;
     int bn = 256, bc = 1, bd = 8, bs = 1;
@@ -1150,21 +1154,28 @@ fo_status autotune(fo_ctx* ctx, Plan& p) {
         Run r;
         fo_status rs = run_product(ctx, p, st, s, "autotune", ci, &r);   // warm-up
         if (rs != FO_OK) { ctx->prof = prof; return rs; }
-        cudaEventRecord(e0, s);
-        for (int rep = 0; rep < kTuneReps; ++rep) {
-            rs = run_product(ctx, p, st, s, "autotune", ci, &r);
-            if (rs != FO_OK) { ctx->prof = prof; return rs; }
-        }
-        cudaEventRecord(e1, s);
         float ms = 0.0f;
-        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-            ctx->prof = prof;
-            return fail(ctx, FO_ERR_CUDA, "autotune timing failed");
+        int reps = kTuneReps;
+        for (int pass = 0; pass < 2; ++pass) {
+            cudaEventRecord(e0, s);
+            for (int rep = 0; rep < reps; ++rep) {
+                rs = run_product(ctx, p, st, s, "autotune", ci, &r);
+                if (rs != FO_OK) { ctx->prof = prof; return rs; }
+            }
+            cudaEventRecord(e1, s);
+            if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+                ctx->prof = prof;
+                return fail(ctx, FO_ERR_CUDA, "autotune timing failed");
+            }
+            ms /= (float)reps;
+            const int want = ms > 0.0f ? (int)std::min((float)kTuneMost, kTuneMs / ms) : kTuneReps;
+            if (want <= reps) break;
+            reps = want;
         }
         if (autotune_log())
             std::fprintf(stderr, "autotune n0=%lld batch=%d tile %dx%dx%d store %d persistent %d: %.4f ms per product\n",
                          (long long)p.key.n[0], p.batch, cands[ci][0], cands[ci][1], cands[ci][2], cands[ci][3],
-                         cands[ci][4], ms / kTuneReps);
+                         cands[ci][4], ms);
         if (best == 0.0f || ms < best) {
             best = ms;
             bn = cands[ci][0];
