@@ -1708,18 +1708,16 @@ fo_status fo_spectral_bounds(fo_ctx* ctx, const double* dH, int64_t n, int64_t l
     if (!dH || !d_bounds || n < 1 || ld < n) return fail(ctx, FO_ERR_ARG, "bad arguments");
     DeviceGuard g(ctx->device);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    PlanKey key;
-    key.n = {n};
-    key.mode = MODE_BOUNDS;
-    Plan* p = nullptr;
-    FO_TRY(get_plan(ctx, key, &p));
-    InstIO io;
-    std::memset(&io, 0, sizeof(io));
-    io.H = dH;
-    io.ldh = ld;
-    FO_CUDA(launch_set_io(&io, 1, p->d_io, p->d_inst, 0, st), "set_io");
-    FO_CUDA(launch_bounds(p->d_inst, p->d_io, 1, p->wg.dev, p->part_g, 0, st), "bounds");
-    FO_CUDA(launch_export_bounds(p->d_res, d_bounds, st), "bounds export");
+    double* part = nullptr;
+    if (n > kBoundsOneMax) {   // the partials live in a plan's workspace
+        PlanKey key;
+        key.n = {n};
+        key.mode = MODE_BOUNDS;
+        Plan* p = nullptr;
+        FO_TRY(get_plan(ctx, key, &p));
+        part = p->part_g;
+    }
+    FO_CUDA(launch_bounds_one(dH, n, ld, part, d_bounds, st), "bounds");
     return FO_OK;
 }
 

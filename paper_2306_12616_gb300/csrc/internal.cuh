@@ -408,7 +408,13 @@ cudaError_t launch_bounds(const Inst* in, const InstIO* io, int batch, Work wg, 
 cudaError_t launch_lanczos(const Inst* in, const InstIO* io, int batch, Work wg, double* part, int steps,
                            cudaStream_t s, int* launches);
 // d_bounds[0..2] = emin, emax, non-finite flag of one instance.
-cudaError_t launch_export_bounds(const DevResult* res, double* out3, cudaStream_t s);
+// Bounds of one matrix to out3 (min, max, non-finite): up to kBoundsOneMax rows in one launch (part
+// is not used), above in two (part: 3 doubles per kGershRows rows). The line is one row per warp of the
+// one launch's cluster (8 blocks of 32 warps): a call takes 14.3 us there at N = 256 and 16.8 in two
+// launches (22 in the four of set-up, rows, reduction and export); with a second row per warp the
+// cluster's 8 SMs fall behind, 19.9 against 16.8 us at N = 384.
+constexpr int64_t kBoundsOneMax = 256;
+cudaError_t launch_bounds_one(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s);
 // X = (2H - (emin+emax) I)/(emax - emin) into slot 0 of every instance.
 cudaError_t launch_scale(const Inst* in, const InstIO* io, Work ws, const Shape& sh, cudaStream_t s,
                          int* dbg);

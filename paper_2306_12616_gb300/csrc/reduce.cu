@@ -8,6 +8,7 @@
 
 #include <cuda.h>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -15,6 +16,8 @@
 #include "fpbits.h"
 #include "internal.cuh"
 #include "tcptx.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace fo {
 namespace {
@@ -85,110 +88,177 @@ __global__ void k_set_io(const IoChunk p, InstIO* d_io, const Inst* insts) {
 // One warp per row: r_i = sum_{j != i} |h_ij| summed exactly (lane-strided 128-bit
 // fixed-point sums merged by a butterfly, rounded to float64 once: csrc/exactsum.h; the
 // float64 adds it replaces bound the kernel on this GPU's narrow float64 pipe), lo_i = h_ii -
-// r_i, hi_i = h_ii + r_i; per-block (min lo, max hi, any non-finite).
+// r_i, hi_i = h_ii + r_i; (min lo, max hi, any non-finite) of warps, blocks and instances, which
+// no order of the reduction changes.
+struct Encl {
+    double lo, hi;
+    int bad;
+};
+__device__ __forceinline__ Encl encl_empty() { return Encl{INFINITY, -INFINITY, 0}; }
+__device__ __forceinline__ void encl_add(Encl& a, const Encl& b) {
+    a.lo = fmin(a.lo, b.lo);
+    a.hi = fmax(a.hi, b.hi);
+    a.bad |= b.bad;
+}
+
+// Row `row` < n of H; lo and hi are the warp's, bad this lane's.
+__device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t n, int64_t ld, int64_t row, int lane) {
+    const unsigned long long* r = reinterpret_cast<const unsigned long long*>(H + row * ld);
+    Encl e = encl_empty();
+    XAcc acc{0, 0, 0};
+    double d = 0.0;
+    // four loads per lane in flight
+    int64_t j = lane;
+    for (; j + 96 < n; j += 128) {
+        uint64_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(r + j + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool fin = ((v[u] >> 52) & 0x7ff) != 0x7ff;
+            e.bad |= !fin;
+            if (j + 32 * u == row) d = __longlong_as_double((long long)v[u]);
+            else if (fin) xacc_add_abs(acc, v[u]);
+        }
+    }
+    for (; j < n; j += 32) {
+        const uint64_t v = __ldg(r + j);
+        const bool fin = ((v >> 52) & 0x7ff) != 0x7ff;
+        e.bad |= !fin;
+        if (j == row) d = __longlong_as_double((long long)v);
+        else if (fin) xacc_add_abs(acc, v);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        XAcc other;
+        other.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
+        other.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
+        other.e = __shfl_xor_sync(0xffffffffu, acc.e, o);
+        xacc_merge(acc, other);
+    }
+    const double s = xacc_to_double(acc);
+    d = warp_sum(d);
+    e.lo = d - s;
+    e.hi = d + s;
+    return e;
+}
+
+// Block reduction of the warps' values (uniform lo and hi within a warp); thread 0 gets the result.
+__device__ __forceinline__ Encl encl_block(Encl e, Encl* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    e.bad = __any_sync(0xffffffffu, e.bad);
+    if (lane == 0) sh[warp] = e;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < nw; ++w) encl_add(e, sh[w]);
+    return e;
+}
+
+// An interval too narrow to divide by is widened to its centre -/+ 1.
+__device__ __forceinline__ void encl_widen(Encl& e) {
+    if (!(e.hi - e.lo > 1e-12 * fmax(1.0, fmax(fabs(e.lo), fabs(e.hi))))) {
+        const double c = 0.5 * (e.lo + e.hi);
+        e.lo = c - 1.0;
+        e.hi = c + 1.0;
+    }
+}
+
+// kGershRows rows from row0 on: the block's partial part[0 .. 2].
+__device__ __forceinline__ void gersh_block(const double* __restrict__ H, int64_t n, int64_t ld, int64_t row0,
+                                            double* part) {
+    __shared__ Encl sh[kGershRows];
+    const int64_t row = row0 + (threadIdx.x >> 5);
+    Encl e = encl_empty();
+    if (row < n) e = gersh_row(H, n, ld, row, threadIdx.x & 31);
+    e = encl_block(e, sh);
+    if (threadIdx.x == 0) {
+        part[0] = e.lo;
+        part[1] = e.hi;
+        part[2] = e.bad ? 1.0 : 0.0;
+    }
+}
+
+// The enclosure from the partials [q0, q1), in thread 0.
+__device__ __forceinline__ Encl gersh_final(const double* part, int q0, int q1) {
+    __shared__ Encl sh[32];
+    Encl e = encl_empty();
+    for (int q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
+        Encl p;
+        p.lo = part[3 * (int64_t)q];
+        p.hi = part[3 * (int64_t)q + 1];
+        p.bad = part[3 * (int64_t)q + 2] != 0.0;
+        encl_add(e, p);
+    }
+    e.lo = warp_min(e.lo);
+    e.hi = warp_max(e.hi);
+    e = encl_block(e, sh);
+    encl_widen(e);
+    return e;
+}
+
 __global__ void __launch_bounds__(32 * kGershRows) k_gershgorin_rows(const Inst* __restrict__ insts,
                                                                      const InstIO* __restrict__ io,
                                                                      Work wg, double* part) {
     pdl_sync();
     const int b = blockIdx.x;
     const int i = inst_of(wg, b);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t n = insts[i].n, ld = io[i].ldh;
-    const double* H = io[i].H;
-    const int64_t row = (int64_t)(b - wg.pre[i]) * kGershRows + warp;
-    double lo = INFINITY, hi = -INFINITY;
-    int bad = 0;
-    if (row < n) {
-        const unsigned long long* r = reinterpret_cast<const unsigned long long*>(H + row * ld);
-        XAcc acc{0, 0, 0};
-        double d = 0.0;
-        // four loads per lane in flight
-        int64_t j = lane;
-        for (; j + 96 < n; j += 128) {
-            uint64_t v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = __ldg(r + j + 32 * u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool fin = ((v[u] >> 52) & 0x7ff) != 0x7ff;
-                bad |= !fin;
-                if (j + 32 * u == row) d = __longlong_as_double((long long)v[u]);
-                else if (fin) xacc_add_abs(acc, v[u]);
-            }
-        }
-        for (; j < n; j += 32) {
-            const uint64_t v = __ldg(r + j);
-            const bool fin = ((v >> 52) & 0x7ff) != 0x7ff;
-            bad |= !fin;
-            if (j == row) d = __longlong_as_double((long long)v);
-            else if (fin) xacc_add_abs(acc, v);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            XAcc other;
-            other.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
-            other.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
-            other.e = __shfl_xor_sync(0xffffffffu, acc.e, o);
-            xacc_merge(acc, other);
-        }
-        const double s = xacc_to_double(acc);
-        d = warp_sum(d);
-        lo = d - s;
-        hi = d + s;
-    }
-    bad = __any_sync(0xffffffffu, bad);
-    __shared__ double slo[kGershRows], shi[kGershRows];
-    __shared__ int sbad[kGershRows];
-    if (lane == 0) { slo[warp] = lo; shi[warp] = hi; sbad[warp] = bad; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double l = slo[0], h = shi[0];
-        int bd = sbad[0];
-        for (int w = 1; w < kGershRows; ++w) {
-            l = fmin(l, slo[w]);
-            h = fmax(h, shi[w]);
-            bd |= sbad[w];
-        }
-        part[3 * (int64_t)b] = l;
-        part[3 * (int64_t)b + 1] = h;
-        part[3 * (int64_t)b + 2] = bd ? 1.0 : 0.0;
-    }
+    gersh_block(io[i].H, insts[i].n, io[i].ldh, (int64_t)(b - wg.pre[i]) * kGershRows, part + 3 * (int64_t)b);
 }
 
 // One block per instance: reduce its partials [pre[i], pre[i+1]).
 __global__ void k_gershgorin_final(const Inst* __restrict__ insts, Work wg, const double* part) {
     pdl_sync();
-    __shared__ double slo[32], shi[32];
-    __shared__ int sbad[32];
     const int i = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double lo = INFINITY, hi = -INFINITY;
-    int bad = 0;
-    for (int q = wg.pre[i] + threadIdx.x; q < wg.pre[i + 1]; q += blockDim.x) {
-        lo = fmin(lo, part[3 * (int64_t)q]);
-        hi = fmax(hi, part[3 * (int64_t)q + 1]);
-        bad |= part[3 * (int64_t)q + 2] != 0.0;
-    }
-    lo = warp_min(lo);
-    hi = warp_max(hi);
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane == 0) { slo[warp] = lo; shi[warp] = hi; sbad[warp] = bad; }
-    __syncthreads();
+    const Encl e = gersh_final(part, wg.pre[i], wg.pre[i + 1]);
     if (threadIdx.x == 0) {
-        for (int w = 1; w < nw; ++w) {
-            lo = fmin(lo, slo[w]);
-            hi = fmax(hi, shi[w]);
-            bad |= sbad[w];
-        }
-        if (!(hi - lo > 1e-12 * fmax(1.0, fmax(fabs(lo), fabs(hi))))) {
-            const double c = 0.5 * (lo + hi);
-            lo = c - 1.0;
-            hi = c + 1.0;
-        }
         DevResult* r = insts[i].res;
-        r->bounds[0] = lo;
-        r->bounds[1] = hi;
-        r->nonfinite = bad;
-        r->status = bad ? FO_ERR_NONFINITE : FO_OK;
+        r->bounds[0] = e.lo;
+        r->bounds[1] = e.hi;
+        r->nonfinite = e.bad;
+        r->status = e.bad ? FO_ERR_NONFINITE : FO_OK;
+    }
+}
+
+// The bounds of one matrix as the caller's three numbers (min, max, 1 if an entry is not finite). The
+// call is bound by its launches (set-up, rows, reduction and export were four of them), so its
+// arguments go to the kernels directly: the rows and their reduction as two launches, or one launch of
+// one cluster, a warp per row and the blocks' values gathered by block 0 through distributed shared memory.
+__global__ void __launch_bounds__(32 * kGershRows) k_bounds_rows(const double* __restrict__ H, int64_t n, int64_t ld,
+                                                                 double* part) {
+    pdl_sync();
+    gersh_block(H, n, ld, (int64_t)blockIdx.x * kGershRows, part + 3 * (int64_t)blockIdx.x);
+}
+__device__ __forceinline__ void store_bounds(const Encl& e, double* out3) {
+    out3[0] = e.lo;
+    out3[1] = e.hi;
+    out3[2] = e.bad ? 1.0 : 0.0;
+}
+__global__ void k_bounds_final(const double* part, int blocks, double* out3) {
+    pdl_sync();
+    const Encl e = gersh_final(part, 0, blocks);
+    if (threadIdx.x == 0) store_bounds(e, out3);
+}
+constexpr int kBoundsCluster = 8;    // portable cluster size
+constexpr int kBoundsThreads = 1024;
+__global__ void __cluster_dims__(kBoundsCluster, 1, 1) __launch_bounds__(kBoundsThreads)
+    k_bounds_cluster(const double* __restrict__ H, int64_t n, int64_t ld, double* out3) {
+    __shared__ Encl sh[kBoundsThreads / 32];
+    __shared__ Encl all[kBoundsCluster];
+    cg::cluster_group cl = cg::this_cluster();
+    pdl_sync();
+    const int rank = (int)cl.block_rank();
+    // consecutive rows on different blocks, so that a small matrix uses all of them
+    Encl e = encl_empty();
+    for (int64_t row = (int64_t)(threadIdx.x >> 5) * kBoundsCluster + rank; row < n;
+         row += (int64_t)(kBoundsThreads / 32) * kBoundsCluster)
+        encl_add(e, gersh_row(H, n, ld, row, threadIdx.x & 31));
+    e = encl_block(e, sh);
+    cl.sync();   // every block has started: block 0's shared memory may be written
+    if (threadIdx.x == 0) *cl.map_shared_rank(&all[rank], 0) = e;
+    cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        for (int b = 1; b < kBoundsCluster; ++b) encl_add(e, all[b]);
+        encl_widen(e);
+        store_bounds(e, out3);
     }
 }
 
@@ -207,13 +277,6 @@ __global__ void k_bounds_given(const Inst* __restrict__ insts, const InstIO* __r
     }
     r->nonfinite = 0;
     r->status = FO_OK;
-}
-
-__global__ void k_export_bounds(const DevResult* res, double* out3) {
-    pdl_sync();
-    out3[0] = res->bounds[0];
-    out3[1] = res->bounds[1];
-    out3[2] = res->nonfinite ? 1.0 : 0.0;
 }
 
 // ------------------------------------------------------------- scaling and splitting
@@ -1163,8 +1226,14 @@ cudaError_t launch_bounds(const Inst* in, const InstIO* io, int batch, Work wg, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_export_bounds(const DevResult* res, double* out3, cudaStream_t s) {
-    launch_pdl(1, k_export_bounds, 1, 1, 0, s, res, out3);
+cudaError_t launch_bounds_one(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s) {
+    if (n <= kBoundsOneMax) {
+        launch_pdl(1, k_bounds_cluster, kBoundsCluster, kBoundsThreads, 0, s, H, n, ld, out3);
+    } else {
+        const int blocks = (int)((n + kGershRows - 1) / kGershRows);
+        launch_pdl(1, k_bounds_rows, blocks, 32 * kGershRows, 0, s, H, n, ld, part);
+        launch_pdl(1, k_bounds_final, 1, 256, 0, s, part, blocks, out3);
+    }
     return cudaGetLastError();
 }
 
