@@ -82,6 +82,34 @@ FO_XS inline void xacc_add_abs(XAcc& a, uint64_t bits) {
     a.hi += thi + (a.lo < tlo ? 1u : 0u);
 }
 
+// acc += |x_0| + ... + |x_{G-1}| for G finite float64 numbers: one rescaling for the group, each term
+// shifted without a branch (lanes of a warp hold entries of very different sizes: the branches of
+// the term-by-term form diverge). A zero adds nothing, whatever its place.
+template <int G>
+FO_XS inline void xacc_add_abs_group(XAcc& a, const uint64_t* bits) {
+    int top = 0;
+    for (int q = 0; q < G; ++q) {
+        const int e = (int)(bits[q] >> 52) & 0x7ff;
+        top = e > top ? e : top;
+    }
+    top = top > 0 ? top : 1;   // subnormals and zeros: biased exponent 1
+    if (top > a.e) {
+        xacc_shr(a, top - a.e);
+        a.e = top;
+    }
+    for (int q = 0; q < G; ++q) {
+        const int f = (int)(bits[q] >> 52) & 0x7ff;
+        const uint64_t m = (bits[q] & 0x000fffffffffffffull) | (f ? 1ull << 52 : 0);
+        // (m : 0) >> r is the term in units of 2^(e - 1133); r >= 6 and m < 2^53
+        const int r = a.e - (f ? f : 1) + 6;
+        const int r2 = r - 64 < 63 ? r - 64 : 63;
+        const uint64_t thi = r < 64 ? m >> r : 0;
+        const uint64_t tlo = r < 64 ? m << (64 - r) : m >> r2;
+        a.lo += tlo;
+        a.hi += thi + (a.lo < tlo ? 1u : 0u);
+    }
+}
+
 // a += b (both accumulators of the same kind of sum)
 FO_XS inline void xacc_merge(XAcc& a, XAcc b) {
     if (b.e > a.e) {

@@ -407,7 +407,6 @@ cudaError_t launch_bounds(const Inst* in, const InstIO* io, int batch, Work wg, 
 // Ritz values widened by their residuals and 1% of the width, clamped to Gershgorin.
 cudaError_t launch_lanczos(const Inst* in, const InstIO* io, int batch, Work wg, double* part, int steps,
                            cudaStream_t s, int* launches);
-// d_bounds[0..2] = emin, emax, non-finite flag of one instance.
 // Bounds of one matrix to out3 (min, max, non-finite): up to kBoundsOneMax rows in one launch (part
 // is not used), above in two (part: 3 doubles per kGershRows rows). The line is one row per warp of the
 // one launch's cluster (8 blocks of 32 warps): a call takes 14.3 us there at N = 256 and 16.8 in two

