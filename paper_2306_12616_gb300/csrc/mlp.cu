@@ -35,8 +35,9 @@ __device__ __forceinline__ float silu_grad_f(float z) {
 // times). The weights' bytes bound it: 145 KB per CTA from L2, about 2300 clocks, as long as the
 // sums of a layer; one CTA per two rows would read all 580 KB. Every sum runs in the order of its
 // definition, one term after another in one thread.
-// One training step of 256 rows, with k_mlp_grad: 16.4 + 13.3 us in 2 launches, where 11 launches
-// took about 205 us (20000 rows, two epochs: 33.5 -> 5.3 ms).
+// One training step of 256 rows, with k_mlp_grad: 2 launches and 31 us, where 11 launches took about
+// 205 us (20000 rows, two epochs: 33.5 -> 4.9 ms; 5.3 while the row indices, targets, biases and Adam's
+// state were requested where they are used and the output sums read eight rows of one bank).
 constexpr int kCl = 4;                          // CTAs per cluster
 constexpr int kRows = 8;                        // rows per cluster
 constexpr int kUnits = kMlpHidden / kCl;        // hidden units per CTA
@@ -80,7 +81,36 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
     const float* B2 = W2 + kMlpHidden * kMlpHidden;
     const float* W3 = B2 + kMlpHidden;
     const float* B3 = W3 + kMlpOut * kMlpHidden;
-    // group 0: the rows and W1; group 1: W2's rows and W3; group 2: W2's columns
+    // this thread: hidden unit u0 + o of rows 2 rg, 2 rg + 1
+    const int o = tid % kUnits, rg = tid / kUnits, r0 = 2 * rg;
+    // what is read once and used late is requested first, ahead of the weights' copies: the rows (through
+    // their indices), the biases and, in the threads of the outputs, their target
+    constexpr int NX = (kRows * kMlpIn + kRowThreads - 1) / kRowThreads;
+    float xv[NX], xm[NX], xs[NX];
+#pragma unroll
+    for (int u = 0; u < NX; ++u) {
+        const int q = tid + u * kRowThreads, rr = q / kMlpIn, i = q - rr * kMlpIn, b = b0 + rr;
+        xv[u] = xm[u] = 0.0f;
+        xs[u] = 1.0f;
+        if (q < kRows * kMlpIn && b < g.B) {
+            xv[u] = g.src[(int64_t)(g.idx ? g.idx[b] : b) * kMlpIn + i];
+            if (g.norm) {
+                xm[u] = g.norm[i];
+                xs[u] = g.norm[kMlpIn + i];
+            }
+        }
+    }
+    const float bias1 = B1[u0 + o], bias2 = B2[u0 + o];
+    float bias3 = 0.0f, t = 0.0f;
+    if (tid < kRows * kMlpOut) {
+        const int rr = tid / kMlpOut, j = tid - rr * kMlpOut, b = b0 + rr;
+        bias3 = B3[j];
+        if (TRAIN && b < g.B) {
+            t = g.tsrc[(int64_t)(g.idx ? g.idx[b] : b) * kMlpOut + j];
+            if (g.norm) t = (t - g.norm[2 * kMlpIn + j]) / g.norm[2 * kMlpIn + kMlpOut + j];
+        }
+    }
+    // group 0: W1; group 1: W2's rows and W3; group 2: W2's columns
     for (int q = tid; q < kUnits * (kMlpIn / 4); q += kRowThreads) {
         const int o = q / (kMlpIn / 4), i = 4 * (q - o * (kMlpIn / 4));
         cp_async16(&sm.w1[o * kLd1 + i], W1 + (u0 + o) * kMlpIn + i);
@@ -99,21 +129,18 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
         }
     }
     cp_async_commit();
-    for (int q = tid; q < kRows * kMlpIn; q += kRowThreads) {
-        const int rr = q / kMlpIn, i = q - rr * kMlpIn, b = b0 + rr;
-        float v = 0.0f;
-        if (b < g.B) {
-            v = g.src[(int64_t)(g.idx ? g.idx[b] : b) * kMlpIn + i];
-            if (g.norm) v = (v - g.norm[i]) / g.norm[kMlpIn + i];
-            if (TRAIN && c == 0) g.x[(int64_t)b * kMlpIn + i] = v;
-        }
+#pragma unroll
+    for (int u = 0; u < NX; ++u) {
+        const int q = tid + u * kRowThreads, rr = q / kMlpIn, i = q - rr * kMlpIn, b = b0 + rr;
+        if (q >= kRows * kMlpIn) break;
+        float v = xv[u];
+        if (g.norm) v = (v - xm[u]) / xs[u];   // (0 past the batch)
+        if (TRAIN && c == 0 && b < g.B) g.x[(int64_t)b * kMlpIn + i] = v;
         sm.x[q] = v;
     }
     cp_async_wait<2>();
     __syncthreads();
     cl.sync();   // every CTA of the cluster runs before its shared memory is written
-    // this thread: hidden unit u0 + o of rows 2 rg, 2 rg + 1
-    const int o = tid % kUnits, rg = tid / kUnits, r0 = 2 * rg;
     auto share = [&](float* dst, float v0, float v1) {   // into every CTA's copy
 #pragma unroll
         for (int q = 0; q < kCl; ++q) {
@@ -144,7 +171,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
         }
     };
     float z10, z11, z20, z21;
-    layer(sm.w1 + o * kLd1, sm.x, kMlpIn, B1[u0 + o], z10, z11);
+    layer(sm.w1 + o * kLd1, sm.x, kMlpIn, bias1, z10, z11);
     {
         const float v0 = silu_f(z10), v1 = silu_f(z11);
         share(sm.a1, v0, v1);
@@ -152,7 +179,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
     }
     cp_async_wait<1>();
     cl.sync();
-    layer(sm.w2r + o * kLd2, sm.a1, kMlpHidden, B2[u0 + o], z20, z21);
+    layer(sm.w2r + o * kLd2, sm.a1, kMlpHidden, bias2, z20, z21);
     {
         const float v0 = silu_f(z20), v1 = silu_f(z21);
         share(sm.a2, v0, v1);
@@ -163,15 +190,20 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
     if (tid < kRows * kMlpOut) {
         // the outputs, in every CTA (the backward pass of each needs them)
         const int rr = tid / kMlpOut, j = tid - rr * kMlpOut, b = b0 + rr;
-        float s = B3[j];
+        float s = bias3;
         const float *w = sm.w3 + j * kMlpHidden, *a = sm.a2 + rr * kMlpHidden;
-#pragma unroll 8
-        for (int i = 0; i < kMlpHidden; ++i) s = fmaf(a[i], w[i], s);
+        // (the eight rows lie in the same banks: one 16-byte read serves four terms)
+#pragma unroll 4
+        for (int i = 0; i < kMlpHidden; i += 4) {
+            const float4 p = *reinterpret_cast<const float4*>(a + i), wv = *reinterpret_cast<const float4*>(w + i);
+            s = fmaf(p.x, wv.x, s);
+            s = fmaf(p.y, wv.y, s);
+            s = fmaf(p.z, wv.z, s);
+            s = fmaf(p.w, wv.w, s);
+        }
         if (b < g.B) {
             if (c == 0) g.y[(int64_t)b * kMlpOut + j] = s;
             if (TRAIN) {
-                float t = g.tsrc[(int64_t)(g.idx ? g.idx[b] : b) * kMlpOut + j];
-                if (g.norm) t = (t - g.norm[2 * kMlpIn + j]) / g.norm[2 * kMlpIn + kMlpOut + j];
                 const float wl = j ? kMlpLossW1 : kMlpLossW0;
                 const float d = s - t;
                 const float dv = 2.0f * wl * d / (float)g.B;
@@ -228,7 +260,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kRowThreads) k_mlp
 // gradient itself or one Adam step of the parameter (Kingma and Ba, bias-corrected, step from 1);
 // one more block adds the loss. A block: kGo outputs x kGi inputs, 128 threads of 1 x 4 parameters;
 // 16 x 32 tiles give 202 blocks for the 152 SMs. Latency bounds it, so dZ and A are requested whole
-// (up to kGb rows) by asynchronous copies before any sum starts (13.3 us; four staged passes took 17).
+// (up to kGb rows) by asynchronous copies before any sum starts (four staged passes took a quarter longer).
 constexpr int kGo = 16, kGi = 32, kGb = 256;
 constexpr int kGradSmem = kGb * (kGo + kGi) * 4;
 constexpr int kTilesI1 = (kMlpIn + 1 + kGi - 1) / kGi, kTilesI2 = (kMlpHidden + 1 + kGi - 1) / kGi;
@@ -309,6 +341,17 @@ __global__ void __launch_bounds__(128) k_mlp_grad(const GradArgs g) {
         s_corr[1] = 1.0f - powf(0.999f, (float)g.step);
     }
     const int o = tid >> 3, i4 = (tid & 7) * 4;
+    // Adam's state of this thread's parameters, requested before the sums
+    float pm[4], pv[4], pp[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = i0 + i4 + u;
+        const int q = i < I ? off + (o0 + o) * I + i : off + O * I + o0 + o;
+        const bool mine = !g.grad && o0 + o < O && i <= I;
+        pm[u] = mine ? g.m[q] : 0.0f;
+        pv[u] = mine ? g.v[q] : 0.0f;
+        pp[u] = mine ? g.p[q] : 0.0f;
+    }
     float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int b0 = 0; b0 < g.B; b0 += kGb) {
         const int nb = g.B - b0 < kGb ? g.B - b0 : kGb;
@@ -354,13 +397,13 @@ __global__ void __launch_bounds__(128) k_mlp_grad(const GradArgs g) {
             g.grad[q] = s[u];
         } else {
             const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-            const float mq = b1 * g.m[q] + (1.0f - b1) * s[u];
-            const float vq = b2 * g.v[q] + (1.0f - b2) * s[u] * s[u];
+            const float mq = b1 * pm[u] + (1.0f - b1) * s[u];
+            const float vq = b2 * pv[u] + (1.0f - b2) * s[u] * s[u];
             g.m[q] = mq;
             g.v[q] = vq;
             const float mh = mq / s_corr[0];
             const float vh = vq / s_corr[1];
-            g.p[q] -= g.lr * mh / (sqrtf(vh) + eps);
+            g.p[q] = pp[u] - g.lr * mh / (sqrtf(vh) + eps);
         }
     }
 }
