@@ -122,6 +122,17 @@ FO_XS inline void xacc_merge(XAcc& a, XAcc b) {
     a.hi += b.hi + (a.lo < b.lo ? 1u : 0u);
 }
 
+// Sums of several accumulators: each brought to the largest exponent first (e >= a.e), then added as
+// 128-bit integers.
+FO_XS inline void xacc_align(XAcc& a, int e) {
+    xacc_shr(a, e - a.e);
+    a.e = e;
+}
+FO_XS inline void xacc_add_aligned(XAcc& a, uint64_t lo, uint64_t hi) {
+    a.lo += lo;
+    a.hi += hi + (a.lo < lo ? 1u : 0u);
+}
+
 // The accumulated sum rounded to float64 (to nearest, ties to even; +inf past the largest
 // finite value).
 FO_XS inline double xacc_to_double(const XAcc& a) {

@@ -86,13 +86,13 @@ __global__ void k_set_io(const IoChunk p, InstIO* d_io, const Inst* insts) {
 
 // ------------------------------------------------------------------ Gershgorin bounds
 // One warp per row: r_i = sum_{j != i} |h_ij| summed exactly (lane-strided 128-bit
-// fixed-point sums merged by a butterfly, rounded to float64 once: csrc/exactsum.h; the
+// fixed-point sums, brought to the warp's largest exponent and added, rounded to float64 once: csrc/exactsum.h; the
 // float64 adds it replaces bound the kernel on this GPU's narrow float64 pipe), lo_i = h_ii -
 // r_i, hi_i = h_ii + r_i; (min lo, max hi, any non-finite) of warps, blocks and instances, which
 // no order of the reduction changes.
 // Integer instructions bound it above N = 1000 (92 us for the 288 MB of N = 6000, 42 of them bytes):
 // terms are added in groups of kGershLoads with one rescaling each and no branches, and as many loads
-// in flight (a bounds call at N = 2048 took 36 us, now 23; 4096 69, now 54; 6000 98, now 92).
+// in flight (a bounds call at N = 2048 took 36 us, now 22.6; 4096 69, now 54; 6000 98, now 92).
 struct Encl {
     double lo, hi;
     int bad;
@@ -127,13 +127,9 @@ __device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t 
         }
         xacc_add_abs_group<kGershLoads>(acc, v);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        XAcc other;
-        other.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
-        other.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
-        other.e = __shfl_xor_sync(0xffffffffu, acc.e, o);
-        xacc_merge(acc, other);
-    }
+    xacc_align(acc, __reduce_max_sync(0xffffffffu, acc.e));
+    for (int o = 16; o > 0; o >>= 1)
+        xacc_add_aligned(acc, __shfl_xor_sync(0xffffffffu, acc.lo, o), __shfl_xor_sync(0xffffffffu, acc.hi, o));
     const double s = xacc_to_double(acc);
     d = warp_sum(d);
     e.lo = d - s;
@@ -141,14 +137,18 @@ __device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t 
     return e;
 }
 
-// Block reduction of the warps' values (uniform lo and hi within a warp); thread 0 gets the result.
+// Block reduction of the warps' values (uniform lo and hi within a warp); warp 0 gets the result.
 __device__ __forceinline__ Encl encl_block(Encl e, Encl* sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     e.bad = __any_sync(0xffffffffu, e.bad);
     if (lane == 0) sh[warp] = e;
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int w = 1; w < nw; ++w) encl_add(e, sh[w]);
+    if (warp == 0) {
+        e = lane < nw ? sh[lane] : encl_empty();
+        e.lo = warp_min(e.lo);
+        e.hi = warp_max(e.hi);
+        e.bad = __any_sync(0xffffffffu, e.bad);
+    }
     return e;
 }
 
@@ -221,6 +221,8 @@ __global__ void k_gershgorin_final(const Inst* __restrict__ insts, Work wg, cons
 // call is bound by its launches (set-up, rows, reduction and export were four of them), so its
 // arguments go to the kernels directly: the rows and their reduction as two launches, or one launch of
 // one cluster, a warp per row and the blocks' values gathered by block 0 through distributed shared memory.
+// On the device the one launch takes 9.4 us at N = 256 and 5.3 at 64 (13.0 and 8.6 while the warps merged
+// sums exponent by exponent and one thread reduced the block), two launches 7.1 at 300; the host 2.6 and 4.1.
 __global__ void __launch_bounds__(32 * kGershRows) k_bounds_rows(const double* __restrict__ H, int64_t n, int64_t ld,
                                                                  double* part) {
     pdl_sync();
@@ -236,7 +238,7 @@ __global__ void k_bounds_final(const double* part, int blocks, double* out3) {
     const Encl e = gersh_final(part, 0, blocks);
     if (threadIdx.x == 0) store_bounds(e, out3);
 }
-constexpr int kBoundsCluster = 8;    // portable cluster size
+constexpr int kBoundsCluster = 8;    // portable cluster size (16 half-sized blocks: 7.6 against 9.4 us at N = 256)
 constexpr int kBoundsThreads = 1024;
 __global__ void __cluster_dims__(kBoundsCluster, 1, 1) __launch_bounds__(kBoundsThreads)
     k_bounds_cluster(const double* __restrict__ H, int64_t n, int64_t ld, double* out3) {
@@ -255,6 +257,7 @@ __global__ void __cluster_dims__(kBoundsCluster, 1, 1) __launch_bounds__(kBounds
     if (threadIdx.x == 0) *cl.map_shared_rank(&all[rank], 0) = e;
     cl.sync();
     if (rank == 0 && threadIdx.x == 0) {
+#pragma unroll
         for (int b = 1; b < kBoundsCluster; ++b) encl_add(e, all[b]);
         encl_widen(e);
         store_bounds(e, out3);

@@ -1,6 +1,7 @@
 """Group sums of csrc/exactsum.h (one rescaling per group, terms shifted without branches) against the
 term-by-term form and math.fsum: the rows of test_exactsum (narrow and wide exponents, zeros,
-subnormals, values near the largest float64), in groups of eight padded with zeros."""
+subnormals, values near the largest float64), in groups of eight padded with zeros; and lane-strided
+sums of groups brought to one exponent and added, as the kernels' warps do."""
 import math
 import os
 import shutil
@@ -36,8 +37,23 @@ int main(int argc, char** argv) {
         XAcc d{0, 0, 0};
         for (int64_t j = 0; j < n; j += 16) xacc_add_abs_group<8>(d, x.data() + j);
         xacc_merge(c, d);
-        double out[3] = {xacc_to_double(a), xacc_to_double(b), xacc_to_double(c)};
-        std::fwrite(out, 8, 3, g);
+        // 32 lane-strided accumulators brought to the largest exponent and added
+        XAcc lane[32], t{0, 0, 0};
+        for (int l = 0; l < 32; ++l) {
+            lane[l] = XAcc{0, 0, 0};
+            for (int64_t j = l; j < n; j += 256) {
+                uint64_t v[8];
+                for (int u = 0; u < 8; ++u) v[u] = j + 32 * u < n ? x[j + 32 * u] : 0;
+                xacc_add_abs_group<8>(lane[l], v);
+            }
+            t.e = lane[l].e > t.e ? lane[l].e : t.e;
+        }
+        for (int l = 0; l < 32; ++l) {
+            xacc_align(lane[l], t.e);
+            xacc_add_aligned(t, lane[l].lo, lane[l].hi);
+        }
+        double out[4] = {xacc_to_double(a), xacc_to_double(b), xacc_to_double(c), xacc_to_double(t)};
+        std::fwrite(out, 8, 4, g);
     }
     std::fclose(f);
     std::fclose(g);
@@ -60,10 +76,10 @@ def test_group_sums_round_like_fsum(tmp_path):
         for x in data:
             f.write(np.int64(len(x)).tobytes() + np.ascontiguousarray(x, dtype=np.float64).tobytes())
     subprocess.run([str(exe), str(fin), str(fout)], check=True)
-    out = np.fromfile(fout).reshape(-1, 3)
+    out = np.fromfile(fout).reshape(-1, 4)
     for x, o in zip(data, out):
         try:
             ref = math.fsum(np.abs(x))
         except OverflowError:
             ref = math.inf
-        assert o[0] == ref and o[1] == ref and o[2] == ref
+        assert np.all(o == ref)
