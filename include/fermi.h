@@ -44,7 +44,10 @@ typedef enum {
     FO_ERR_UNSUPPORTED = 8       /* feature not available for these arguments */
 } fo_status;
 
-/* Arithmetic of the matrix products. FP64 runs everything in float64. The split forms
+/* Arithmetic of the matrix products. FP64: float64 matrices; each product is formed from eight
+ * signed 8-bit digits per entry, whose products are summed exactly on the tensor cores and
+ * rounded to float64 once (as accurate as float64 FMAs; those run instead for FO_FLAG_STAGED and
+ * where the digit buffers, 48 bytes per entry and the partial sums, do not fit the device). The split forms
  * keep float32 master copies of every matrix and run each product on the tensor cores
  * as a sum of products of 16-bit planes with float32 accumulation:
  *   BF16X3: A = a0 + a1 + a2 (bf16 planes), AB ~ sum_{i+j<=2} a_i b_j  (6 products)

@@ -5,7 +5,7 @@
 // arithmetic). Each stage of the method is one launch over the whole batch: a kernel
 // finds its instance either from blockIdx.y (stages with the same work per instance) or
 // from a per-instance prefix sum of block counts (stages whose work grows with the
-// instance size: the block-to-instance map is a binary search on the prefix).
+// instance size: the block-to-instance map is a table, or for a few instances a search on the prefix).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -445,7 +445,7 @@ __global__ void k_diag_sums(const Inst* __restrict__ insts, int is64) {
 // --------------------------------------------------------- Frobenius inner products
 // <S_{giant0+g}, S_{baby0+b}>_F of one instance. Every matrix is symmetric, so the product is
 // the diagonal sum plus twice the strict upper triangle: only the chunks (kChunk consecutive
-// entries of one row) on or above the diagonal are read. A block covers kGChunks consecutive
+// entries of one row) on or above the diagonal are read. A block covers gram_chunks consecutive
 // upper chunks. They are copied kCPS chunks at a time into a kGStages-deep shared-memory ring
 // by cp.async (16 bytes per copy, no register staging; each thread's copy addresses are
 // fixed up front and only offset per chunk), matrix-major (row s of a chunk holds the chunk
@@ -463,7 +463,7 @@ __global__ void k_diag_sums(const Inst* __restrict__ insts, int is64) {
 // left of the diagonal. Every lane sums at most kGChunks * kChunk / 32 products per pair in
 // T; lanes are combined by shuffles in T and blocks by the float64 partial sums (k_sum_partials).
 constexpr int kChunkBytes = 512;    // one chunk of one matrix: 128 float32 / 64 float64
-constexpr int kGChunks = 64;        // chunks per block
+constexpr int kGChunks = 64;        // most chunks per block (gram_chunks)
 constexpr int kCPS = 2;             // chunks per stage
 constexpr int kGStages = 4;         // shared-memory ring depth (stages)
 constexpr int kMaxRows = 48;        // staged rows (giant and baby groups, padded)
