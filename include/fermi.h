@@ -173,7 +173,8 @@ typedef struct {
     int32_t evals;            /* evaluations of P (1 unless FO_MU_LEARNED corrected mu) */
     int32_t order;            /* expansion order proposed by the learned model (FO_MU_LEARNED) or
                                  the coefficients used (FO_MU_ORDER); 0 otherwise */
-    int32_t tile_drain;       /* accumulator drain warps of the product kernel (0 for FP64) */
+    int32_t tile_drain;       /* accumulator drain warps of the product kernel (0 for FP64); the
+                                 autotuner may pick 16 with 128-wide tiles too */
     int32_t tile_store;       /* operand plane storage used (1 or 2 as in fo_params; 0 for FP64) */
     double  trace_raw;        /* tr(P) as the expansion produced it, before the trace correction
                                  (equal to trace when none was applied) */

@@ -1136,9 +1136,9 @@ fo_status autotune(fo_ctx* ctx, Plan& p) {
     // mirrored epilogue writes for transposed operand loads: it pays on short tiles), and the
     // persistent kernel (128-wide tiles; its epilogue overlaps the next tile's products)
     const int cands[12][5] = {{256, 1, 8, 1, 0}, {256, 1, 16, 1, 0}, {128, 1, 8, 1, 0}, {128, 2, 8, 1, 0},
-                              {128, 1, 8, 1, 1}, {256, 1, 8, 2, 0}, {256, 1, 16, 2, 0}, {128, 1, 8, 2, 0},
-                              {128, 2, 8, 2, 0}, {128, 1, 8, 2, 1}};
-    const int ncand = p.key.sym ? 10 : 5;
+                              {128, 1, 8, 1, 1}, {128, 1, 16, 1, 0}, {256, 1, 8, 2, 0}, {256, 1, 16, 2, 0},
+                              {128, 1, 8, 2, 0}, {128, 2, 8, 2, 0}, {128, 1, 8, 2, 1}, {128, 1, 16, 2, 0}};
+    const int ncand = p.key.sym ? 12 : 6;
     int bp = 0;
     for (int ci = 0; ci < ncand; ++ci) {
         // the persistent kernel is timed only when asked for: measured slower on every workload
@@ -1146,6 +1146,7 @@ fo_status autotune(fo_ctx* ctx, Plan& p) {
         // co-resident CTAs do)
         if (p.key.persist_req != 2 && cands[ci][4]) continue;
         if (p.key.persist_req == 2 && !cands[ci][4]) continue;
+        if (p.chain && cands[ci][0] == 128 && cands[ci][2] == 16) continue;   // not built for chain launches
         p.tile_n = cands[ci][0];
         p.tile_ctas = cands[ci][1];
         p.tile_drain = cands[ci][2];
