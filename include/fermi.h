@@ -46,8 +46,13 @@ typedef enum {
 
 /* Arithmetic of the matrix products. FP64: float64 matrices; each product is formed from eight
  * signed 8-bit digits per entry, whose products are summed exactly on the tensor cores and
- * rounded to float64 once (as accurate as float64 FMAs; those run instead for FO_FLAG_STAGED and
- * where the digit buffers, 48 bytes per entry and the partial sums, do not fit the device). The split forms
+ * rounded to float64 once. Its error is that of float64 FMAs norm-wise: relative to the largest
+ * entries of the operands, whose common exponent all digits share. It is not entry-wise: an entry
+ * 2^-40 of the largest keeps about three digits, so that a block of P that couples two fragments by
+ * 1e-8 of the largest entry is good to about 1e-10 of itself (1e-12: 1e-6) where FMAs give 1e-15.
+ * FO_FLAG_FP64_FMA asks for the FMAs, which keep small entries' own relative accuracy and take 8 to
+ * 40 times as long; they also run for FO_FLAG_STAGED and where the digit buffers, 48 bytes per entry
+ * and the partial sums, do not fit the device. The split forms
  * keep float32 master copies of every matrix and run each product on the tensor cores
  * as a sum of products of 16-bit planes with float32 accumulation:
  *   BF16X3: A = a0 + a1 + a2 (bf16 planes), AB ~ sum_{i+j<=2} a_i b_j  (6 products)
@@ -94,6 +99,10 @@ typedef enum {
                                           with m > k: the longer Clenshaw chain, ~1.4e-6 at
                                           m = 50); without this flag they fail with
                                           FO_ERR_UNSUPPORTED */
+#define FO_FLAG_FP64_FMA         0x80u /* FO_PREC_FP64: form the products by float64 FMAs instead of
+                                          digit products (see fo_precision): for callers who need
+                                          the relative accuracy of entries far below the largest.
+                                          No effect on the split forms */
 #define FO_FLAG_STAGED           0x8u  /* baby and giant steps in the staged form of Algorithm 1
                                           (Sec. "Speed up with multiple GPU streams"): the
                                           independent products of a stage in one launch, about

@@ -17,7 +17,7 @@ from dataclasses import dataclass
 __all__ = [
     "FO_OK", "FO_PREC_FP64", "FO_PREC_BF16X3", "FO_PREC_FP16X2", "FO_PREC_BF16X1",
     "FO_MU_FIXED", "FO_MU_BISECT", "FO_MU_LEARNED", "FO_MU_ORDER", "FO_FLAG_NO_RESULT_SYNC", "FO_FLAG_GRAPH",
-    "FO_FLAG_STAGED", "FO_FLAG_POWER_BASIS", "FO_FLAG_NO_TRACE_FIX", "FO_FLAG_ALLOW_LOOSE",
+    "FO_FLAG_STAGED", "FO_FLAG_POWER_BASIS", "FO_FLAG_NO_TRACE_FIX", "FO_FLAG_ALLOW_LOOSE", "FO_FLAG_FP64_FMA",
     "FoParams", "FoResult", "FermiError", "lib", "library_path", "EXPORTED_SYMBOLS",
     "fo_create", "fo_destroy", "fo_last_error", "fo_status_string", "fo_version",
     "fo_spectral_bounds", "fo_chebyshev_coeffs", "fo_density_matrix", "fo_density_matrix_host",
@@ -40,6 +40,7 @@ FO_FLAG_STAGED = 0x8
 FO_FLAG_POWER_BASIS = 0x10
 FO_FLAG_NO_TRACE_FIX = 0x20
 FO_FLAG_ALLOW_LOOSE = 0x40
+FO_FLAG_FP64_FMA = 0x80
 
 PRECISIONS = {"fp64": FO_PREC_FP64, "bf16x3": FO_PREC_BF16X3, "fp16x2": FO_PREC_FP16X2,
               "bf16x1": FO_PREC_BF16X1}

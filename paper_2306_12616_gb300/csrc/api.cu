@@ -35,6 +35,7 @@ struct PlanKey {
     int mode = MODE_DENSITY, n_terms = 1, k_req = 0, prec = 0, mu_mode = 0, n_quad = 0;
     int use_given = 0, tile_req = 0, ctas_req = 0, drain_req = 0, store_req = 0, sym = 1, max_bisect = 0, max_newton = 0, staged = 0, lanczos = 0, power = 0, nofix = 0;
     int chain = 0, chain_win = 0, persist_req = 0;
+    int fma64 = 0;   // float64 products by FMAs although the digit products could form them
     double tr_tol = 0.0;
     bool operator==(const PlanKey& o) const {
         return n == o.n && mode == o.mode && n_terms == o.n_terms && k_req == o.k_req && prec == o.prec &&
@@ -42,7 +43,8 @@ struct PlanKey {
                tile_req == o.tile_req && ctas_req == o.ctas_req && drain_req == o.drain_req &&
                store_req == o.store_req && sym == o.sym && max_bisect == o.max_bisect &&
                max_newton == o.max_newton && tr_tol == o.tr_tol && staged == o.staged && lanczos == o.lanczos && power == o.power &&
-               nofix == o.nofix && chain == o.chain && chain_win == o.chain_win && persist_req == o.persist_req;
+               nofix == o.nofix && chain == o.chain && chain_win == o.chain_win && persist_req == o.persist_req &&
+               fma64 == o.fma64;
     }
 };
 
@@ -391,8 +393,8 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     }
     for (Bucket& bk : p->buckets) bk.off = take((size_t)bk.inst_bytes * bk.count);
     // float64 plans whose chains run step by step: digit buffers (staged chains multiply arbitrary
-    // pairs of slots and keep the FMA kernel)
-    p->digits = digits && sh.is64 && !key.staged && (key.mode == MODE_DENSITY || key.mode == MODE_MOMENTS);
+    // pairs of slots and keep the FMA kernel), unless the caller asks for the FMAs
+    p->digits = digits && sh.is64 && !key.staged && !key.fma64 && (key.mode == MODE_DENSITY || key.mode == MODE_MOMENTS);
     if (p->digits) {
         std::vector<int64_t> ns, nps;
         for (const Inst& in : p->inst) {
@@ -1337,6 +1339,7 @@ fo_status density_batch(fo_ctx* ctx, int batch, const double* const* dH, const i
     key.chain = prm->chain;
     key.chain_win = prm->chain_window;
     key.persist_req = prm->tile_persist;
+    key.fma64 = prm->precision == FO_PREC_FP64 && (prm->flags & FO_FLAG_FP64_FMA) ? 1 : 0;
     if (prm->mu_mode == FO_MU_LEARNED) {
         key.max_newton = prm->max_newton;
         key.tr_tol = prm->tr_tol;
@@ -1574,6 +1577,7 @@ fo_status features_batch(fo_ctx* ctx, int batch, const double* const* dH, const 
     key.max_bisect = q.max_bisect;
     key.staged = (prm->flags & FO_FLAG_STAGED) ? 1 : 0;
     key.lanczos = q.lanczos_steps;
+    key.fma64 = q.precision == FO_PREC_FP64 && (prm->flags & FO_FLAG_FP64_FMA) ? 1 : 0;
     Plan* p = nullptr;
     FO_TRY(get_plan(ctx, key, &p));
     std::vector<InstIO> io(batch);

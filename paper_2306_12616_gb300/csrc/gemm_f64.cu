@@ -1,6 +1,7 @@
 // Float64 recurrence product out = alpha * A B + beta * C + D + shift * I_n on the float64 FMA pipe:
-// the float64 path of staged chains, and of plans whose digit buffers do not fit the device
-// (elsewhere gemm_digits.cu, 8 to 40 times faster at N = 256 ... 2000).
+// the float64 path of staged chains, of plans whose digit buffers do not fit the device, and of
+// callers who need small entries' relative accuracy (FO_FLAG_FP64_FMA); elsewhere gemm_digits.cu,
+// 8 to 40 times faster at N = 256 ... 2000.
 //
 // 64 x 64 output
 // tiles, 16-deep k slices staged in shared memory, 4 x 4 outputs per thread. The update of
