@@ -397,8 +397,10 @@ __global__ void __launch_bounds__(128) k_mlp_grad(const GradArgs g) {
             g.grad[q] = s[u];
         } else {
             const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-            const float mq = b1 * pm[u] + (1.0f - b1) * s[u];
-            const float vq = b2 * pv[u] + (1.0f - b2) * s[u] * s[u];
+            // the products that are rounded by themselves, written out: left to the compiler, constant
+            // b1 and b2 moved the contraction to the other product
+            const float mq = fmaf(b1, pm[u], (1.0f - b1) * s[u]);
+            const float vq = fmaf(b2, pv[u], (1.0f - b2) * s[u] * s[u]);
             g.m[q] = mq;
             g.v[q] = vq;
             const float mh = mq / s_corr[0];
