@@ -109,7 +109,7 @@ constexpr int kMuNodes = 32;        // nodes per thread held in shared memory (u
 struct MuNodes {
     double e[kMuNodes][32], w[kMuNodes][32];
 };
-__device__ __forceinline__ void trace_at(double mu, const MuNodes& nd, const double* __restrict__ w,
+__device__ __forceinline__ void trace_at(double mu, const MuNodes& nd, const double* w,
                                          const double* __restrict__ ct, int M, double mid, double half, double inv2kT,
                                          double (*sh)[2 * kMuCluster], int& par, int rank, double* tr, double* dtr) {
     cg::cluster_group cl = cg::this_cluster();
@@ -168,7 +168,7 @@ __device__ __forceinline__ void trace_at(double mu, const MuNodes& nd, const dou
 // the bracket is narrower than 1e-15 (emax - emin) (mu = midpoint), at most max_iter
 // evaluations.
 __global__ void __cluster_dims__(kMuCluster, 1, 1) __launch_bounds__(32) k_bisect(const Inst* __restrict__ insts,
-                                                 const InstIO* __restrict__ io,
+                                                 const InstIO* io,
                                                  const double* __restrict__ ct, int M,
                                                  int max_iter, int start_mu0) {
     pdl_sync();
@@ -254,7 +254,7 @@ __global__ void __cluster_dims__(kMuCluster, 1, 1) __launch_bounds__(32) k_bisec
 }
 
 // mu of FO_MU_FIXED from the per-call inputs.
-__global__ void k_set_mu(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int batch) {
+__global__ void k_set_mu(const Inst* __restrict__ insts, const InstIO* io, int batch) {
     pdl_sync();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch) insts[i].res->mu = io[i].mu;
@@ -262,7 +262,7 @@ __global__ void k_set_mu(const Inst* __restrict__ insts, const InstIO* __restric
 
 // f_j = f(e_j; mu) at the nodes e_j = mid + half x_j, mu read from the device record.
 // Block (node chunk, instance).
-__global__ void k_fermi_nodes(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int M,
+__global__ void k_fermi_nodes(const Inst* __restrict__ insts, const InstIO* io, int M,
                               const double* __restrict__ ct) {
     pdl_sync();
     const Inst& in = insts[blockIdx.y];
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(256) k_contract_f64(const Inst* __restrict__ i
         for (int t = 1; t < k; ++t) {
             double v[kCtRows];
 #pragma unroll
-            for (int u = 0; u < kCtRows; ++u) v[u] = __ldg(tbase + (int64_t)(t - 1) * tstride + (int64_t)(8 * u) * np);
+            for (int u = 0; u < kCtRows; ++u) v[u] = tbase[(int64_t)(t - 1) * tstride + (int64_t)(8 * u) * np];
 #pragma unroll
             for (int q = 0; q < kGroup; ++q) {
                 const double g = l0 + q < m ? gsh[(l0 + q) * k + t] : 0.0;

@@ -473,7 +473,7 @@ struct DigStep {
 // per entry of the square, about half of them from L2): the float64 pipe sees one or two
 // operations per entry (alpha is a power of two, folded into the conversion; magnitudes are
 // compared as integers).
-__global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __restrict__ insts, const InstIO* __restrict__ io,
+__global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __restrict__ insts, const InstIO* io,
                                                     Work ws, const DigStep st) {
     pdl_sync();
     __shared__ double sv[32][33];
@@ -516,10 +516,10 @@ __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __r
     }
     for (int s = 0; s < sl; ++s, lo0 += kT * kT)
 #pragma unroll
-        for (int q = 0; q < kUpCols; ++q) lo[q] += __ldg(lo0 + o[q]);
+        for (int q = 0; q < kUpCols; ++q) lo[q] += lo0[o[q]];
     for (int s = 0; s < shi; ++s, hi0 += kT * kT)
 #pragma unroll
-        for (int q = 0; q < kUpCols; ++q) hi[q] += __ldg(hi0 + o[q]);
+        for (int q = 0; q < kUpCols; ++q) hi[q] += hi0[o[q]];
     if (cg == 0) {
         // the scales: warp 0, a lane per k range
         const int ea = in.sexp[st.a], eb = in.sexp[st.b];

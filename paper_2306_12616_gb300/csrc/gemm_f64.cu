@@ -21,7 +21,7 @@ constexpr int BM = 64, BN = 64, BK = 16;
 // (b mod tiles) - pre[i] of instance i for step b / tiles.
 __global__ void __launch_bounds__(256) k_gemm_f64(const __grid_constant__ StepList steps,
                                                   const Inst* __restrict__ insts,
-                                                  const InstIO* __restrict__ io, Work wt) {
+                                                  const InstIO* io, Work wt) {
     __shared__ double As[BK][BM + 1];
     __shared__ double Bs[BK][BN];
     const int sidx = blockIdx.x / wt.total;

@@ -233,7 +233,7 @@ template <int PA, int PB, int NPROD, bool F16, int TBN, int MINB, int DW, bool C
 __global__ void __launch_bounds__(32 * (2 + DW), MINB)
     k_tc_gemm(const __grid_constant__ TcMaps maps,
               const __grid_constant__ std::conditional_t<CHAIN, ChainList, StepList> steps,
-              const Inst* __restrict__ insts, const InstIO* __restrict__ io, const int* __restrict__ pre,
+              const Inst* __restrict__ insts, const InstIO* io, const int* __restrict__ pre,
               const uint2* __restrict__ tab, int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag) {
     using Cfg = TcCfg<PA, PB, NPROD, F16, TBN, MINB, DW>;
     constexpr int S = Cfg::kStages;
@@ -1076,7 +1076,7 @@ __device__ __forceinline__ void persist_tile(int t, int tiles, int tile0, const 
 // partials of a float64-output product.
 template <bool F16, int EW, int TBN, int LD>
 __device__ __forceinline__ void persist_epilogue(const Step& st, const Inst* __restrict__ insts,
-                                                 const InstIO* __restrict__ io, int inst, int m0, int n0, int sym,
+                                                 const InstIO* io, int inst, int m0, int n0, int sym,
                                                  bool ub, float* tile, double (*rowpart)[2], int ew, int lane) {
     const Inst& in = insts[inst];
     const int64_t n_real = in.n;
@@ -1267,7 +1267,7 @@ __device__ __forceinline__ void persist_epilogue(const Step& st, const Inst* __r
 template <int PA, int PB, int NPROD, bool F16, int DW, int EW>
 __global__ void __launch_bounds__(32 * (2 + DW + EW), 1)
     k_tc_persist(const __grid_constant__ TcMaps maps, const __grid_constant__ StepList steps,
-                 const Inst* __restrict__ insts, const InstIO* __restrict__ io, const int* __restrict__ pre,
+                 const Inst* __restrict__ insts, const InstIO* io, const int* __restrict__ pre,
                  int i0, int i1, int tile0, int tiles, int b0, int sym, int* err_flag) {
     using Cfg = PcCfg<PA, PB, NPROD, F16, DW, EW>;
     constexpr int S = Cfg::kStages;

@@ -168,6 +168,11 @@ struct Work {
 // visible (and, since that one waited the same way, everything before it): every kernel launched
 // this way executes it, in all threads, before it touches global memory other than the plan's
 // constant tables, and holds nothing then that another kernel's blocks could be waiting for.
+// Its lifetime begins before its predecessors have written, so it reads only those constant tables
+// (Inst, prefixes, block and tile tables, cosines) through the read-only path: everything else (H,
+// InstIO, slots, partial sums, records) by plain loads. __ldg and const __restrict__ parameters
+// promise data that does not change while the kernel runs, and the compiler may move them across
+// the wait.
 // Waiting blocks are not free: they share the SM of what still runs. The network's training kernels
 // (5.2 -> 5.7 ms for two epochs) and the kernel behind the Frobenius products are launched plainly.
 // Measured with this on all others: N = 64 1.04 -> 0.91 ms, N = 1000 2.02 -> 1.91 ms.

@@ -97,7 +97,7 @@ __global__ void k_lz_init(const Inst* __restrict__ insts, int batch) {
 // they are used, in the order the sums take them (one load at a time kept 2 KB per warp in flight:
 // 15.7 us per step at N = 1501, 12.3 now).
 __global__ void __launch_bounds__(32 * kGershRows) k_lz_matvec(const Inst* __restrict__ insts,
-                                                               const InstIO* __restrict__ io, Work wg, int j,
+                                                               const InstIO* io, Work wg, int j,
                                                                double* part) {
     pdl_sync();
     __shared__ double sp[kGershRows];
@@ -116,14 +116,14 @@ __global__ void __launch_bounds__(32 * kGershRows) k_lz_matvec(const Inst* __res
         for (; c + 32 * (kLzLoads - 1) < n; c += 32 * kLzLoads) {
             double hv[kLzLoads], qv[kLzLoads];
 #pragma unroll
-            for (int u = 0; u < kLzLoads; ++u) hv[u] = __ldg(hr + c + 32 * u);
+            for (int u = 0; u < kLzLoads; ++u) hv[u] = hr[c + 32 * u];
 #pragma unroll
             for (int u = 0; u < kLzLoads; ++u) qv[u] = z.q[c + 32 * u];
 #pragma unroll
             for (int u = 0; u < kLzLoads; ++u) s = fma(hv[u], qv[u], s);
         }
 #pragma unroll 4
-        for (; c < n; c += 32) s = fma(__ldg(hr + c), z.q[c], s);
+        for (; c < n; c += 32) s = fma(hr[c], z.q[c], s);
         s = warp_sum_d(s);
         const double wv = s - z.beta[j] * z.qp[row];
         if (lane == 0) z.w[row] = wv;

@@ -440,7 +440,7 @@ __global__ void k_col_stats(const float* __restrict__ X, int n, int C, float* __
 
 // Features of every instance (row = caller index when rows_by_user, else plan order):
 // tau_1..tau_64 / n (tau_j, j > 2k, zero), N_e / n, 2 kT / (e_b - e_a), e_a / 100, e_b / 100.
-__global__ void k_features(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int batch, int k,
+__global__ void k_features(const Inst* __restrict__ insts, const InstIO* io, int batch, int k,
                            int rows_by_user, float* __restrict__ feat) {
     const int i = blockIdx.x, c = threadIdx.x;
     if (i >= batch || c >= kMlpIn) return;
@@ -530,7 +530,7 @@ __global__ void k_learned_mu(const Inst* __restrict__ insts, int batch, const fl
 // expansion, k_poly_width, which is kT for an exact Fermi function) or a secant step
 // through the previous evaluation, limited to 10 kT_p; else leave the instance active for
 // the bisection fallback.
-__global__ void k_learned_check(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int batch,
+__global__ void k_learned_check(const Inst* __restrict__ insts, const InstIO* io, int batch,
                                 int round, int max_rounds, double tol, int is64, int* __restrict__ active_count) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch) return;

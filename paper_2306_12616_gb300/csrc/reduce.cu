@@ -106,7 +106,7 @@ __device__ __forceinline__ void encl_add(Encl& a, const Encl& b) {
 }
 
 // Row `row` < n of H; lo and hi are the warp's, bad this lane's.
-__device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t n, int64_t ld, int64_t row, int lane) {
+__device__ __forceinline__ Encl gersh_row(const double* H, int64_t n, int64_t ld, int64_t row, int lane) {
     const unsigned long long* r = reinterpret_cast<const unsigned long long*>(H + row * ld);
     Encl e = encl_empty();
     XAcc acc{0, 0, 0};
@@ -116,7 +116,7 @@ __device__ __forceinline__ Encl gersh_row(const double* __restrict__ H, int64_t 
     for (int64_t j = lane; j < n; j += 32 * kGershLoads) {
         uint64_t v[kGershLoads];
 #pragma unroll
-        for (int u = 0; u < kGershLoads; ++u) v[u] = j + 32 * u < n ? __ldg(r + j + 32 * u) : 0;
+        for (int u = 0; u < kGershLoads; ++u) v[u] = j + 32 * u < n ? r[j + 32 * u] : 0;
 #pragma unroll
         for (int u = 0; u < kGershLoads; ++u) {
             const bool fin = ((v[u] >> 52) & 0x7ff) != 0x7ff;
@@ -162,7 +162,7 @@ __device__ __forceinline__ void encl_widen(Encl& e) {
 }
 
 // kGershRows rows from row0 on: the block's partial part[0 .. 2].
-__device__ __forceinline__ void gersh_block(const double* __restrict__ H, int64_t n, int64_t ld, int64_t row0,
+__device__ __forceinline__ void gersh_block(const double* H, int64_t n, int64_t ld, int64_t row0,
                                             double* part) {
     __shared__ Encl sh[kGershRows];
     const int64_t row = row0 + (threadIdx.x >> 5);
@@ -195,7 +195,7 @@ __device__ __forceinline__ Encl gersh_final(const double* part, int q0, int q1) 
 }
 
 __global__ void __launch_bounds__(32 * kGershRows) k_gershgorin_rows(const Inst* __restrict__ insts,
-                                                                     const InstIO* __restrict__ io,
+                                                                     const InstIO* io,
                                                                      Work wg, double* part) {
     pdl_sync();
     const int b = blockIdx.x;
@@ -223,7 +223,7 @@ __global__ void k_gershgorin_final(const Inst* __restrict__ insts, Work wg, cons
 // one cluster, a warp per row and the blocks' values gathered by block 0 through distributed shared memory.
 // On the device the one launch takes 9.4 us at N = 256 and 5.3 at 64 (13.0 and 8.6 while the warps merged
 // sums exponent by exponent and one thread reduced the block), two launches 7.1 at 300; the host 2.6 and 4.1.
-__global__ void __launch_bounds__(32 * kGershRows) k_bounds_rows(const double* __restrict__ H, int64_t n, int64_t ld,
+__global__ void __launch_bounds__(32 * kGershRows) k_bounds_rows(const double* H, int64_t n, int64_t ld,
                                                                  double* part) {
     pdl_sync();
     gersh_block(H, n, ld, (int64_t)blockIdx.x * kGershRows, part + 3 * (int64_t)blockIdx.x);
@@ -241,7 +241,7 @@ __global__ void k_bounds_final(const double* part, int blocks, double* out3) {
 constexpr int kBoundsCluster = 8;    // portable cluster size (16 half-sized blocks: 7.6 against 9.4 us at N = 256)
 constexpr int kBoundsThreads = 1024;
 __global__ void __cluster_dims__(kBoundsCluster, 1, 1) __launch_bounds__(kBoundsThreads)
-    k_bounds_cluster(const double* __restrict__ H, int64_t n, int64_t ld, double* out3) {
+    k_bounds_cluster(const double* H, int64_t n, int64_t ld, double* out3) {
     __shared__ Encl sh[kBoundsThreads / 32];
     __shared__ Encl all[kBoundsCluster];
     cg::cluster_group cl = cg::this_cluster();
@@ -265,7 +265,7 @@ __global__ void __cluster_dims__(kBoundsCluster, 1, 1) __launch_bounds__(kBounds
 }
 
 // Given bounds (InstIO emin/emax) or bounds copied from device memory (bounds_src).
-__global__ void k_bounds_given(const Inst* __restrict__ insts, const InstIO* __restrict__ io, int batch) {
+__global__ void k_bounds_given(const Inst* __restrict__ insts, const InstIO* io, int batch) {
     pdl_sync();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch) return;
@@ -324,7 +324,7 @@ __device__ __forceinline__ void store_split(float v, float* x, uint16_t* p, int6
 // (the float64 pipe of this GPU is narrow: one multiply per entry; the rounding to float32 is
 // done with integer operations).
 __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ insts,
-                                                   const InstIO* __restrict__ io, Work ws,
+                                                   const InstIO* io, Work ws,
                                                    const Shape sh, int* dbg) {
     pdl_sync();
     __shared__ double tile[32][33];
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(256) k_scale_sym(const Inst* __restrict__ inst
     }
 }
 
-__global__ void k_pack_f32(const float* __restrict__ A, int64_t n, int64_t lda, char* slot, int64_t np,
+__global__ void k_pack_f32(const float* A, int64_t n, int64_t lda, char* slot, int64_t np,
                            int planes, int fp16, float pscale) {
     pdl_sync();
     const int64_t total = np * np;
@@ -1033,7 +1033,7 @@ __global__ void __launch_bounds__(64) k_assemble_moments(const Inst* __restrict_
 // ------------------------------------------------------------ trace and ||P||_F^2
 // Block = red_rows(np) rows of one instance's P; partials (tr, ||.||^2) per block.
 __global__ void __launch_bounds__(256) k_trace_frob_part(const Inst* __restrict__ insts,
-                                                         const InstIO* __restrict__ io, Work we,
+                                                         const InstIO* io, Work we,
                                                          double* partials) {
     pdl_sync();
     __shared__ double sh[33];
@@ -1109,7 +1109,7 @@ __global__ void k_trace_frob_final(const Inst* __restrict__ insts, Work we, cons
 //    diagonal entries when the correction was applied and |r| <= 1e-4 max(1, N_e) (a larger
 //    residual is left in place for the caller to see) and sums the new diagonal for the
 //    reported trace.
-__global__ void k_tile_trace(const Inst* __restrict__ insts, const InstIO* __restrict__ io, const int* pre,
+__global__ void k_tile_trace(const Inst* __restrict__ insts, const InstIO* io, const int* pre,
                              const double* part, int mode) {
     pdl_sync();
     __shared__ double sh[33];
@@ -1172,7 +1172,7 @@ __global__ void k_tile_trace(const Inst* __restrict__ insts, const InstIO* __res
 }
 
 // P = R_0 (m = 1): slot n_tslots to the instance's float64 P.
-__global__ void k_copy_out(const Inst* __restrict__ insts, const InstIO* __restrict__ io, Work we,
+__global__ void k_copy_out(const Inst* __restrict__ insts, const InstIO* io, Work we,
                            int slot, int is64) {
     pdl_sync();
     const int i = inst_of(we, blockIdx.x);
