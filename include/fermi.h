@@ -141,8 +141,10 @@ typedef struct {
                                  Gershgorin interval. Not a guaranteed enclosure; ignored with
                                  use_given_bounds */
     int32_t tile_drain;       /* warps draining the tensor-memory accumulators: 0 = autotune,
-                                 8, or 16 (with tile_n = 256); set together with tile_n;
-                                 other values fail with FO_ERR_ARG */
+                                 8, or 16 (with tile_n = 256, or with tile_n = 128, one CTA per
+                                 SM and one launch per product: tile_ctas = 2, tile_persist = 2
+                                 and chain = 2 have 8); set together with tile_n; other values
+                                 fail with FO_ERR_ARG */
     int32_t tile_store;       /* storage of the 16-bit operand planes of the split forms' matrix
                                  slots: 0 = chosen with the tile (autotuned with tile_n = 0,
                                  else 1); 1 = the full square (the symmetric products mirror
@@ -182,8 +184,8 @@ typedef struct {
     int32_t evals;            /* evaluations of P (1 unless FO_MU_LEARNED corrected mu) */
     int32_t order;            /* expansion order proposed by the learned model (FO_MU_LEARNED) or
                                  the coefficients used (FO_MU_ORDER); 0 otherwise */
-    int32_t tile_drain;       /* accumulator drain warps of the product kernel (0 for FP64); the
-                                 autotuner may pick 16 with 128-wide tiles too */
+    int32_t tile_drain;       /* accumulator drain warps of the product kernel (0 for FP64); with
+                                 tile_n and tile_ctas it can be asked for as reported */
     int32_t tile_store;       /* operand plane storage used (1 or 2 as in fo_params; 0 for FP64) */
     double  trace_raw;        /* tr(P) as the expansion produced it, before the trace correction
                                  (equal to trace when none was applied) */

@@ -1093,7 +1093,7 @@ fo_status run_density(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run) {
 }
 
 // Tile configuration of the tensor-core products: the requested one, or the fastest of
-// (256 wide, 1 CTA/SM, 8 or 16 drain warps), (128 wide, 1 CTA/SM) and (128 wide, 2 CTAs/SM)
+// (256 or 128 wide, 1 CTA/SM, 8 or 16 drain warps) and (128 wide, 2 CTAs/SM, 8)
 // on this plan's first baby step, timed with CUDA events on the plan's own layout (the data
 // are whatever the workspace holds; the work does not depend on them).
 fo_status autotune(fo_ctx* ctx, Plan& p) {
@@ -1254,8 +1254,10 @@ fo_status check_params(fo_ctx* ctx, const fo_params* prm) {
         return fail(ctx, FO_ERR_ARG, "tile_n must be 0, 128 or 256");
     if (prm->tile_drain != 0 && (prm->tile_drain != 8 && prm->tile_drain != 16))
         return fail(ctx, FO_ERR_ARG, "tile_drain must be 0, 8 or 16");
-    if (prm->tile_drain == 16 && prm->tile_n != 256)
-        return fail(ctx, FO_ERR_ARG, "16 drain warps need tile_n = 256");
+    if (prm->tile_drain == 16 && prm->tile_n != 256 &&
+        (prm->tile_n != 128 || prm->tile_ctas == 2 || prm->tile_persist == 2 || prm->chain == 2))
+        return fail(ctx, FO_ERR_ARG,
+                    "16 drain warps need tile_n = 256, or tile_n = 128 with one CTA per SM and one launch per product");
     if ((prm->flags & FO_FLAG_POWER_BASIS) && prm->precision == FO_PREC_FP16X2)
         return fail(ctx, FO_ERR_UNSUPPORTED, "the power basis overflows the fp16 range");
     if (prm->precision != FO_PREC_FP64 && !(prm->flags & FO_FLAG_ALLOW_LOOSE)) {
