@@ -22,6 +22,7 @@
 #include <string>
 #include <vector>
 
+#include "gramsplit.h"
 #include "internal.cuh"
 
 using namespace fo;
@@ -412,9 +413,11 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     // per-instance float64 arrays
     std::vector<size_t> small(batch);
     const int ndiag = sh.n_tslots + 2;
+    const int gram_per = gram_chunks(npad.data(), batch, sh.is64);
     for (int j = 0; j < batch; ++j) {
         Inst& in = p->inst[j];
-        in.gram_blocks = gram_blocks_for(in.np, sh.is64);
+        in.gram_per = gram_per;
+        in.gram_blocks = gram_blocks_for(in.np, sh.is64, gram_per);
         size_t o = off;
         o += align256(8 * (size_t)sh.km);             // c
         o += align256(8 * (size_t)sh.km);             // g

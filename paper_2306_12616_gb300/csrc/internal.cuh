@@ -71,6 +71,7 @@ struct Inst {
     int32_t bucket;       // tensor-map bucket (instances of equal np)
     int32_t in_bucket;    // index within the bucket
     int32_t gram_blocks;  // blocks of the Frobenius-product kernel for this instance
+    int32_t gram_per;     // chunks per block (gramsplit.h)
     int32_t user;         // index of the instance in the caller's arrays
     // float64 products on the tensor cores (gemm_digits.cu); null / 0 elsewhere
     char* dig;            // kDigBufs digit buffers of 16 np^2 bytes
@@ -464,7 +465,7 @@ cudaError_t launch_copy_out(const Inst* in, const InstIO* io, Work we, const Sha
 cudaError_t launch_pack_f32(const float* A, int64_t n, int64_t lda, char* slot, int64_t np, int planes,
                             int fp16, float pscale, cudaStream_t s);
 // Blocks of the Frobenius-product kernel for one instance (upper-triangle chunks).
-int gram_blocks_for(int64_t np, int is64);
+int gram_blocks_for(int64_t np, int is64, int per);
 
 // ------------------------------------------------------------------- mlp.cu
 // Learned chemical potential: 68 inputs (64 moments, N_e/N, kT_x, e_a/100, e_b/100),

@@ -14,6 +14,7 @@
 
 #include "exactsum.h"
 #include "fpbits.h"
+#include "gramsplit.h"
 #include "internal.cuh"
 #include "tcptx.cuh"
 
@@ -445,7 +446,7 @@ __global__ void k_diag_sums(const Inst* __restrict__ insts, int is64) {
 // --------------------------------------------------------- Frobenius inner products
 // <S_{giant0+g}, S_{baby0+b}>_F of one instance. Every matrix is symmetric, so the product is
 // the diagonal sum plus twice the strict upper triangle: only the chunks (kChunk consecutive
-// entries of one row) on or above the diagonal are read. A block covers gram_chunks consecutive
+// entries of one row) on or above the diagonal are read. A block covers gram_per consecutive
 // upper chunks. They are copied kCPS chunks at a time into a kGStages-deep shared-memory ring
 // by cp.async (16 bytes per copy, no register staging; each thread's copy addresses are
 // fixed up front and only offset per chunk), matrix-major (row s of a chunk holds the chunk
@@ -462,8 +463,6 @@ __global__ void k_diag_sums(const Inst* __restrict__ insts, int is64) {
 // once at the end); the diagonal chunk of a row weighs them by 1, 1/2 or 0 right of, on or
 // left of the diagonal. Every lane sums at most kGChunks * kChunk / 32 products per pair in
 // T; lanes are combined by shuffles in T and blocks by the float64 partial sums (k_sum_partials).
-constexpr int kChunkBytes = 512;    // one chunk of one matrix: 128 float32 / 64 float64
-constexpr int kGChunks = 64;        // most chunks per block (gram_chunks)
 constexpr int kCPS = 2;             // chunks per stage
 constexpr int kGStages = 4;         // shared-memory ring depth (stages)
 constexpr int kMaxRows = 48;        // staged rows (giant and baby groups, padded)
@@ -477,21 +476,6 @@ __host__ __device__ inline int gram_threads(int ntiles, int tpw) {
     int w = (ntiles + tpw - 1) / tpw;
     if (w < kGramMinThreads / 32) w = kGramMinThreads / 32;
     return 32 * w;
-}
-
-// Upper chunks of an np x np matrix: row r holds chunks floor(r / kc) .. np / kc - 1.
-__host__ __device__ inline int64_t upper_chunks(int64_t np, int kc) {
-    const int64_t cpr = np / kc;
-    return (int64_t)kc * cpr * (cpr + 1) / 2;
-}
-
-// Chunks per block. float32: kGChunks (the partial sums' grouping is part of the result's bits).
-// float64: as few as give an instance about 300 blocks, since the float64 FMAs bound the kernel and a
-// small matrix would otherwise use few SMs (N = 256: 10 blocks of 64 chunks, 0.35 ms).
-__host__ __device__ inline int gram_chunks(int64_t np, bool is64) {
-    if (!is64) return kGChunks;
-    const int64_t c = upper_chunks(np, kChunkBytes / 8) / 300;
-    return c < 2 ? 2 : (c > kGChunks ? kGChunks : (int)c);
 }
 
 template <typename T, int TG, int TB, int TPW>
@@ -513,7 +497,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const Inst* __restrict
     const int64_t np = in.np;
     const int64_t cpr = np / kChunk;                  // chunks per row
     const int64_t nchunks = upper_chunks(np, kChunk);
-    const int per = gram_chunks(np, sizeof(T) == 8);
+    const int per = in.gram_per;
     const int64_t c0 = (int64_t)lb * per;
     const int64_t c1 = c0 + per < nchunks ? c0 + per : nchunks;
     const int ngq = (ngiant + TG - 1) / TG, nbq = (nbaby + TB - 1) / TB;
@@ -1257,9 +1241,8 @@ cudaError_t launch_diag_sums(const Inst* in, int batch, int count, const Shape& 
     return cudaGetLastError();
 }
 
-int gram_blocks_for(int64_t np, int is64) {
+int gram_blocks_for(int64_t np, int is64, int per) {
     const int64_t u = upper_chunks(np, kChunkBytes / (is64 ? 8 : 4));
-    const int per = gram_chunks(np, is64 != 0);
     return (int)((u + per - 1) / per);
 }
 
