@@ -420,6 +420,8 @@ cudaError_t launch_lanczos(const Inst* in, const InstIO* io, int batch, Work wg,
 // cluster's 8 SMs fall behind, 19.9 against 16.8 us at N = 384.
 constexpr int64_t kBoundsOneMax = 256;
 cudaError_t launch_bounds_one(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s);
+// The two-launch form at any size.
+cudaError_t launch_bounds_two(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s);
 // X = (2H - (emin+emax) I)/(emax - emin) into slot 0 of every instance.
 cudaError_t launch_scale(const Inst* in, const InstIO* io, Work ws, const Shape& sh, cudaStream_t s,
                          int* dbg);

@@ -1212,14 +1212,16 @@ cudaError_t launch_bounds(const Inst* in, const InstIO* io, int batch, Work wg, 
     return cudaGetLastError();
 }
 
+cudaError_t launch_bounds_two(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s) {
+    const int blocks = (int)((n + kGershRows - 1) / kGershRows);
+    launch_pdl(1, k_bounds_rows, blocks, 32 * kGershRows, 0, s, H, n, ld, part);
+    launch_pdl(1, k_bounds_final, 1, 256, 0, s, part, blocks, out3);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_bounds_one(const double* H, int64_t n, int64_t ld, double* part, double* out3, cudaStream_t s) {
-    if (n <= kBoundsOneMax) {
-        launch_pdl(1, k_bounds_cluster, kBoundsCluster, kBoundsThreads, 0, s, H, n, ld, out3);
-    } else {
-        const int blocks = (int)((n + kGershRows - 1) / kGershRows);
-        launch_pdl(1, k_bounds_rows, blocks, 32 * kGershRows, 0, s, H, n, ld, part);
-        launch_pdl(1, k_bounds_final, 1, 256, 0, s, part, blocks, out3);
-    }
+    if (n > kBoundsOneMax) return launch_bounds_two(H, n, ld, part, out3, s);
+    launch_pdl(1, k_bounds_cluster, kBoundsCluster, kBoundsThreads, 0, s, H, n, ld, out3);
     return cudaGetLastError();
 }
 
