@@ -160,8 +160,8 @@ struct fo_ctx {
     cudaStream_t cap = nullptr;   // stream for graph capture
     bool capturing = false;
     int* hcount = nullptr;        // pinned readback of the learned judge's active count
-    // learned-mu model (device, float32): parameters, gradients, Adam moments, normalisation
-    float* mlp = nullptr;         // params | grad | m | v | norm
+    // learned-mu model (device, float32): parameters, Adam moments, normalisation
+    float* mlp = nullptr;         // params | m | v | norm
     bool mlp_ready = false;       // trained, loaded or set
     int mlp_step = 0;             // Adam steps taken
     float* mlp_scratch = nullptr; // training buffers
@@ -439,11 +439,11 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     }
     const size_t off_res = take(sizeof(DevResult) * batch);
     // work lists
-    auto fill = [&](HostWork& w, auto count) {
+    auto fill = [&](HostWork& w, auto count, bool table = true) {   // table: the kernels read it (inst_of)
         w.pre.assign(batch + 1, 0);
         for (int j = 0; j < batch; ++j) w.pre[j + 1] = w.pre[j] + (int)count(p->inst[j]);
         w.tab.clear();
-        if (batch > kSmallBatch)
+        if (table && batch > kSmallBatch)
             for (int j = 0; j < batch; ++j) w.tab.insert(w.tab.end(), w.pre[j + 1] - w.pre[j], j);
     };
     fill(p->wg, [](const Inst& in) { return (in.n + kGershRows - 1) / kGershRows; });
@@ -453,8 +453,8 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     fill(p->wgr, [](const Inst& in) { return (int64_t)in.gram_blocks; });
     fill(p->wct, [&](const Inst& in) { return (int64_t)ct_blocks(in.np, sh.k); });
     const bool full = key.mode == MODE_PRODUCT && !key.sym;
-    fill(p->wtc[0], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 256) : tc_tiles(in.np, 256); });
-    fill(p->wtc[1], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 128) : tc_tiles(in.np, 128); });
+    fill(p->wtc[0], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 256) : tc_tiles(in.np, 256); }, false);
+    fill(p->wtc[1], [&](const Inst& in) { return full ? tc_tiles_full(in.np, 128) : tc_tiles(in.np, 128); }, false);
     for (int q = 0; q < 2 && !sh.is64; ++q) {
         // the tiles of the two work lists, in their order: row blocks, and within them the column
         // tiles that reach the diagonal (all of them for a product that is not symmetric)
@@ -468,7 +468,8 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
         }
     }
     fill(p->wf64, [](const Inst& in) { return f64_tiles(in.np); });
-    fill(p->wdig, [&](const Inst& in) { return p->digits ? dig_units(in.np, in.dig_sl, in.dig_sh) : int64_t(0); });
+    fill(p->wdig, [&](const Inst& in) { return p->digits ? dig_units(in.np, in.dig_sl, in.dig_sh) : int64_t(0); },
+         false);
     const size_t off_pg = take(8 * 3 * (size_t)std::max(1, p->wg.pre[batch]));
     const size_t off_pt = take(8 * 2 * (size_t)std::max(1, p->wr.pre[batch]));
     const size_t off_ptc = take(8 * 2 * (size_t)std::max(1, p->wtc[1].pre[batch]));   // 128-blocks
@@ -572,6 +573,7 @@ fo_status place_plan(fo_ctx* ctx, Plan* p) {
             w->dev.tab = reinterpret_cast<const int*>(reinterpret_cast<char*>(p->dtab) + o);
             std::memcpy(host.data() + o, w->tab.data(), sizeof(int) * w->tab.size());
             o += align256(sizeof(int) * w->tab.size());
+            w->tab = std::vector<int>();   // only the device copy is used
         }
     }
     for (int q = 0; q < 2; ++q) {
@@ -983,7 +985,7 @@ fo_status evaluate(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int poly_trac
     h = prof_begin(ctx, s, FO_STAGE_CONTRACT);
     lstage = sh.is64 ? 1 : (sh.m + 31) / 32 + (sh.m > 1 ? 1 : 0);   // + the plane mirror of R_{m-1}
     if (p.digits && sh.m > 1) FO_CUDA(dig_reset(p.d_inst, p.batch, sh.n_tslots, sh.m, s), "digit records");
-    FO_CUDA(launch_contract(p.d_inst, p.we.dev, p.wct.dev, p.wsc.dev, sh, s, ctx->flag + 1), "contract");
+    FO_CUDA(launch_contract(p.d_inst, p.wct.dev, p.wsc.dev, sh, s, ctx->flag + 1), "contract");
     if (p.digits && sh.m > 1) {
         FO_CUDA(dig_split(p.d_inst, p.wsc.dev, sh.n_tslots, sh.m, dig_buf(p, sh.n_tslots), s), "digits of R");
         lstage += 2;
@@ -998,6 +1000,12 @@ fo_status evaluate(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int poly_trac
     return trace_stage(ctx, p, s, run, tmode);
 }
 
+size_t mlp_floats() { return 3 * (size_t)mlp_offsets().total + kMlpNorm; }
+float* mlp_params(fo_ctx* ctx) { return ctx->mlp; }
+float* mlp_m(fo_ctx* ctx) { return ctx->mlp + (size_t)mlp_offsets().total; }
+float* mlp_v(fo_ctx* ctx) { return ctx->mlp + 2 * (size_t)mlp_offsets().total; }
+float* mlp_norm(fo_ctx* ctx) { return ctx->mlp + 3 * (size_t)mlp_offsets().total; }
+
 // Learned mu: moments up to 2k from the baby steps, the network's proposal, evaluation of P
 // and the trace judge; corrected re-evaluations; exact moments and bisection for whatever
 // is still rejected. Eager calls stop as soon as every instance is accepted; a captured
@@ -1007,9 +1015,8 @@ fo_status evaluate(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int poly_trac
 fo_status propose(fo_ctx* ctx, Plan& p, cudaStream_t s, Run* run, int use_order) {
     const Shape& sh = p.sh;
     const int B = p.batch;
-    const MlpOffsets mo = mlp_offsets();
     const float* params = ctx->mlp;
-    const float* norm = ctx->mlp + 4 * (size_t)mo.total;
+    const float* norm = mlp_norm(ctx);
     float* feat = p.lscratch;
     float* y = feat + (size_t)B * kMlpIn;
     int h = prof_begin(ctx, s, FO_STAGE_MOMENTS);
@@ -1476,12 +1483,6 @@ fo_status density_batch(fo_ctx* ctx, int batch, const double* const* dH, const i
 }
 
 // ---------------------------------------------------------------- learned model
-size_t mlp_floats() { return 4 * (size_t)mlp_offsets().total + kMlpNorm; }
-float* mlp_params(fo_ctx* ctx) { return ctx->mlp; }
-float* mlp_m(fo_ctx* ctx) { return ctx->mlp + 2 * (size_t)mlp_offsets().total; }
-float* mlp_v(fo_ctx* ctx) { return ctx->mlp + 3 * (size_t)mlp_offsets().total; }
-float* mlp_norm(fo_ctx* ctx) { return ctx->mlp + 4 * (size_t)mlp_offsets().total; }
-
 fo_status ensure_mlp(fo_ctx* ctx) {
     if (ctx->mlp) return FO_OK;
     if (cudaMalloc(&ctx->mlp, sizeof(float) * mlp_floats()) != cudaSuccess) {

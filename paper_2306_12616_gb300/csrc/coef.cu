@@ -805,7 +805,7 @@ cudaError_t launch_g_to_d(const Inst* in, int batch, const Shape& sh, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const Shape& sh, cudaStream_t s, int* dbg) {
+cudaError_t launch_contract(const Inst* in, Work wct, Work wsym, const Shape& sh, cudaStream_t s, int* dbg) {
     if (sh.is64) {
         const size_t smem = ((size_t)sh.k * sh.m + 32 * 33) * sizeof(double);
         if (smem > 48 * 1024)

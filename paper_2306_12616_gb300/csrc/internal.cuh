@@ -539,7 +539,7 @@ cudaError_t launch_bisect(const Inst* in, const InstIO* io, int batch, const Sha
 cudaError_t launch_set_mu(const Inst* in, const InstIO* io, int batch, cudaStream_t s);
 cudaError_t launch_coefficients(const Inst* in, const InstIO* io, int batch, const Shape& sh,
                                 const double* ct, int with_poly_trace, cudaStream_t s, int* launches);
-cudaError_t launch_contract(const Inst* in, Work we, Work wct, Work wsym, const Shape& sh, cudaStream_t s, int* dbg);
+cudaError_t launch_contract(const Inst* in, Work wct, Work wsym, const Shape& sh, cudaStream_t s, int* dbg);
 // g -> the paper's power-basis coefficients d (in place), for the Horner evaluation.
 cudaError_t launch_g_to_d(const Inst* in, int batch, const Shape& sh, cudaStream_t s);
 

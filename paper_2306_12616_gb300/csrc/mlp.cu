@@ -55,7 +55,7 @@ struct RowSmem {
     float a1[kRows * kMlpHidden];
     float a2[kRows * kMlpHidden];
     float dz2[kRows * kMlpHidden];
-    float y[kRows * kMlpOut], dy[kRows * kMlpOut];
+    float dy[kRows * kMlpOut];
 };
 
 struct RowArgs {
