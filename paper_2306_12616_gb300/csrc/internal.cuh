@@ -176,7 +176,7 @@ struct Work {
 // the wait.
 // Waiting blocks are not free: they share the SM of what still runs. The network's training kernels
 // (5.2 -> 5.7 ms for two epochs) and the kernel behind the Frobenius products are launched plainly.
-// Measured with this on all others: N = 64 1.04 -> 0.91 ms, N = 1000 2.02 -> 1.91 ms.
+// Measured with this on all others: N = 64 1.04 -> 0.87 ms, N = 1000 2.03 -> 1.93 ms.
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_sync() {
@@ -185,7 +185,14 @@ __device__ __forceinline__ void pdl_sync() {
 }
 // Of small-batch launches (launch_pdl with a batch), the kernels between the products are dependent
 // programmatically only up to this many instances: beyond it they are long enough to hide a launch,
-// and what waits beside them costs more (512 instances: 34.9 -> 35.9 ms).
+// and what waits beside them costs more. The block tables and the block size of the DOS weights have the
+// same line. Whole calls with it at infinity against at 0, BF16x3, 300 terms, per count of instances:
+//   N = 64    1: 739 / 767 us   4: 788 / 795   5: 796 / 801   6: 802 / 796   8: 827 / 804   64: 1360 / 1038
+//   N = 256   1: 896 / 923      4: 944 / 961   5: 957 / 966   6: 977 / 966   8: 1009 / 981  64: 2065 / 1739
+//   N = 1000  1: 1572 / 1583    4: 1806 / 1807 5: 2539 / 2542 6: 2638 / 2627 8: 2828 / 2799 16: 5437 / 5362
+// and FP64 at N = 256: 1: 1509 / 1599, 2: 1939 / 1912, 4: 2452 / 2451, 6: 2889 / 2875, 16: 3793 / 3676.
+// The sides cross between 5 and 6 at every size, but for FP64 at 2. (Replayed as a CUDA graph, plain
+// launches are 1 to 4 % faster at any of these counts: a graph exposes less launch latency.)
 constexpr int kSmallBatch = 4;
 template <class... P, class... A>
 cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
