@@ -55,6 +55,7 @@
 #include <vector>
 #include <type_traits>
 
+#include "digits.h"
 #include "internal.cuh"
 #include "tcptx.cuh"
 
@@ -69,7 +70,6 @@ constexpr int kRing = kLowStages * 4 * kBoxBytes;   // 192 KB, the same for both
 constexpr int kMmaSmem = kRing + 1024 /*align*/ + 256 /*barriers*/;
 constexpr int kDrainWarps = 8;                // 64 accumulator columns each
 constexpr int kMmaThreads = 32 * (2 + kDrainWarps);
-constexpr int kPoison = 1 << 20;            // exponent of a matrix holding an infinity or a NaN
 
 static_assert(kHighStages * 2 * kBoxBytes == kRing, "ring of the high orders");
 static_assert(kMmaSmem <= 232448 - 64, "shared memory of the unit kernel");
@@ -91,24 +91,6 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
 }
 // kind::f16, float32 accumulators, float16 operands, both K-major, M = N = 128
 constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kT >> 3) << 17) | ((uint32_t)(kT >> 4) << 24);
-
-// The accumulator restarts: accumulator a's groups of k16 blocks (8 for the low orders, whose
-// largest has 8 pairs: 64 MMAs; 16 for the high orders, at most 4 pairs) are shifted by a quarter
-// group each. gs = log2 of a quarter group. begins / ends: whether block l of cnt starts / ends a
-// group of accumulator a.
-__host__ __device__ constexpr bool acc_begins(int a, int l, int gs) {
-    return l == 0 || ((l + (a << gs)) & ((4 << gs) - 1)) == 0;
-}
-__host__ __device__ constexpr bool acc_ends(int a, int l, int cnt, int gs) {
-    return l == cnt - 1 || ((l + 1 + (a << gs)) & ((4 << gs) - 1)) == 0;
-}
-// The accumulator issued q-th in block l: one that ends there first, one that begins there last.
-__host__ __device__ constexpr int acc_order(int q, int l, int gs) {
-    const int qm = (1 << gs) - 1;
-    if (((l + 1) & qm) == 0) return ((4 - (((l + 1) >> gs) & 3)) + q) & 3;
-    if ((l & qm) == 0 && l > 0) return ((4 - ((l >> gs) & 3)) + 1 + q) & 3;
-    return q;
-}
 
 // The O + 1 digit pairs of order O for one k16 block.
 template <int O>
@@ -269,14 +251,14 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
                 }
                 fence_after();
                 const uint32_t alo = (uint32_t)desc0 + (uint32_t)s * SB, blo = alo + NBX * (kBoxBytes >> 4);
-                // the block's place in the groups' period, as a constant: every accumulator index, start
+                // the block's phase in the groups' period, as a constant: every accumulator index, start
                 // and end is then static (with run-time ones an accumulator switch took ~140 clocks)
                 bool go = true;
                 auto block = [&](auto ph_tag) {
                     constexpr int PH = decltype(ph_tag)::value;
                     auto acc_step = [&](auto q_tag) {
-                        constexpr int A = acc_order(decltype(q_tag)::value, PH == 0 ? (4 << GS) : PH, GS);
-                        constexpr bool BEG = acc_begins(A, PH == 0 ? (4 << GS) : PH, GS);
+                        constexpr int A = acc_order(decltype(q_tag)::value, acc_place(PH, GS), GS);
+                        constexpr bool BEG = acc_begins(A, acc_place(PH, GS), GS);
                         constexpr bool END = acc_ends(A, PH, 1 << 30, GS);
                         if (BEG && l > 0 && go) {
                             go = mbar_wait_warp(&seg_empty[A], (par >> A) & 1u, kWaitNs, vabort);
@@ -377,28 +359,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
 
 // ------------------------------------------------------------------ scales and digits
 
-// An e with b < 0.99 2^e (kPoison when b is not finite); any e serves a zero matrix.
-__device__ __forceinline__ int scale_exp(double b) {
-    if (!(b <= 1.7e308)) return kPoison;
-    if (b < 1e-290) return -960;
-    return ilogb(b * (1.0 / 0.989)) + 1;
-}
-
-// The digits of x at scale 2^e (|x| < 0.99 2^e) as the bytes d_i + 128, d_0 in the top byte: x
-// 2^(63-e) rounded to an integer below 0.99 2^63, plus 128 at every byte.
-__device__ __forceinline__ unsigned long long digits_of(double x, int e) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7ff);
-    const unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
-    const int sh = (ex ? ex : 1) - 1012 - e;
-    unsigned long long v;
-    if (sh >= 0) v = m << (sh < 10 ? sh : 10);
-    else if (sh > -55) v = (m + (1ull << (-sh - 1))) >> -sh;
-    else v = 0;
-    if ((long long)b < 0) v = 0ull - v;
-    return v + 0x8080808080808080ull;
-}
-
 // The eight digits of eight consecutive columns of one row (bytes as above) into the digit
 // buffer: 16 bytes of float16 integers per digit.
 __device__ __forceinline__ void store_digits(char* dig, int64_t np, int64_t row, int64_t col,
@@ -422,38 +382,6 @@ __device__ __forceinline__ void store_digits(char* dig, int64_t np, int64_t row,
         }
         *reinterpret_cast<uint4*>(dst + p * 32) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-}
-
-// (hi 2^32 + lo) 2^(e - 70) rounded to float64, to nearest even.
-__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
-    unsigned long long l = ((unsigned long long)hi << 32) + (unsigned long long)lo;
-    unsigned long long h = (unsigned long long)((hi >> 32) + (lo >> 63)) + (l < (unsigned long long)lo ? 1ull : 0ull);
-    const unsigned long long sign = h & 0x8000000000000000ull;
-    if (sign) {
-        l = 0ull - l;
-        h = ~h + (l == 0ull ? 1ull : 0ull);
-    }
-    if ((h | l) == 0ull) return 0.0;
-    const int lz = h ? __clzll((long long)h) : 64 + __clzll((long long)l);
-    unsigned long long m, rest;   // the leading 64 bits, and what is left below them
-    if (lz == 0) {
-        m = h;
-        rest = l;
-    } else if (lz < 64) {
-        m = (h << lz) | (l >> (64 - lz));
-        rest = l << lz;
-    } else {
-        m = l << (lz - 64);
-        rest = 0;
-    }
-    unsigned long long r = m >> 11;
-    const unsigned long long low = m & 0x7ffull;
-    r += (low > 0x400ull || (low == 0x400ull && (rest != 0ull || (r & 1ull)))) ? 1ull : 0ull;
-    const int E = 127 - lz + e - 70 + 1023;   // biased exponent of the leading bit
-    if (E > 0 && E < 2046)
-        return __longlong_as_double((long long)((((unsigned long long)E << 52) + (r - (1ull << 52))) | sign));
-    const double v = scalbn((double)r, E - 1023 - 52);
-    return sign ? -v : v;
 }
 
 constexpr int kUpWarps = 16, kUpCols = 32 / kUpWarps;
