@@ -394,8 +394,10 @@ fo_status layout_plan(fo_ctx* ctx, const PlanKey& key, Plan* p, bool digits) {
     }
     for (Bucket& bk : p->buckets) bk.off = take((size_t)bk.inst_bytes * bk.count);
     // float64 plans whose chains run step by step: digit buffers (staged chains multiply arbitrary
-    // pairs of slots and keep the FMA kernel), unless the caller asks for the FMAs
-    p->digits = digits && sh.is64 && !key.staged && !key.fma64 && (key.mode == MODE_DENSITY || key.mode == MODE_MOMENTS);
+    // pairs of slots and keep the FMA kernel), unless the caller asks for the FMAs or there is no
+    // product (one moment or two, one term: the digits of X would be formed for nothing, 5 us)
+    const bool products = (key.mode == MODE_DENSITY && (sh.k > 1 || sh.m > 1)) || (key.mode == MODE_MOMENTS && sh.k > 1);
+    p->digits = digits && sh.is64 && products && !key.staged && !key.fma64;
     if (p->digits) {
         std::vector<int64_t> ns, nps;
         for (const Inst& in : p->inst) {
