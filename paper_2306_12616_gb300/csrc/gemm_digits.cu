@@ -442,12 +442,13 @@ __global__ void __launch_bounds__(32 * kUpWarps, 3) k_dig_update(const Inst* __r
         cv[q] = C ? C[mo] : 0.0;
         dv[q] = D ? D[mo] : 0.0;
     }
+    // (streaming loads: each sum is read once; through L1 as other data the product takes 0.4 % longer)
     for (int s = 0; s < sl; ++s, lo0 += kT * kT)
 #pragma unroll
-        for (int q = 0; q < kUpCols; ++q) lo[q] += lo0[o[q]];
+        for (int q = 0; q < kUpCols; ++q) lo[q] += __ldcs(lo0 + o[q]);
     for (int s = 0; s < shi; ++s, hi0 += kT * kT)
 #pragma unroll
-        for (int q = 0; q < kUpCols; ++q) hi[q] += hi0[o[q]];
+        for (int q = 0; q < kUpCols; ++q) hi[q] += __ldcs(hi0 + o[q]);
     if (cg == 0) {
         // the scales: warp 0, a lane per k range
         const int ea = in.sexp[st.a], eb = in.sexp[st.b];
