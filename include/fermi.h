@@ -51,8 +51,9 @@ typedef enum {
  * 2^-40 of the largest keeps about three digits, so that a block of P that couples two fragments by
  * 1e-8 of the largest entry is good to about 1e-10 of itself (1e-12: 1e-6) where FMAs give 1e-15.
  * FO_FLAG_FP64_FMA asks for the FMAs, which keep small entries' own relative accuracy; a call then
- * takes 5 to 6 times as long at N = 20 to 64, 14 at 1000, 34 at 5000. They also run for FO_FLAG_STAGED and where the digit buffers, 48 bytes per entry
- * and the partial sums, do not fit the device. The split forms
+ * takes 5 to 6 times as long at N = 20 to 64, 14 at 1000, 34 at 5000. They also run for
+ * FO_FLAG_STAGED and where the digit buffers, 48 bytes per entry and the partial sums, do not fit
+ * the device. The split forms
  * keep float32 master copies of every matrix and run each product on the tensor cores
  * as a sum of products of 16-bit planes with float32 accumulation:
  *   BF16X3: A = a0 + a1 + a2 (bf16 planes), AB ~ sum_{i+j<=2} a_i b_j  (6 products)
